@@ -553,6 +553,36 @@ qmc_status build_tables(qmc_wf* wf) {
     exp_tab[2 * j + 1] = (float)(v - (long double)exp_tab[2 * j]);
   }
 
+  // ---- small-molecule path (small_eval.cuh): MO rows in canonical shell order,
+  // scaled exponents, 2^(j/2048)
+  bool all_sp = true;
+  d.any_sto = 0;
+  std::vector<double> nak((size_t)d.n_shell * QMC_MAX_PRIM, 0.0);
+  for (int q = 0; q < d.n_shell; ++q) {
+    all_sp = all_sp && (shells[q].canon == 1 || shells[q].canon == 2);
+    if (shells[q].kind == 0) d.any_sto = 1;
+    for (int k = 0; k < shells[q].n_prim; ++k)
+      nak[(size_t)q * QMC_MAX_PRIM + k] = (double)(-2048.0L * (long double)shells[q].expo[k] / 0.6931471805599453094L);
+  }
+  std::vector<double> mo64c((size_t)nao * nmo);
+  for (int b = 0; b < nao; ++b)
+    for (int m = 0; m < nmo; ++m) mo64c[(size_t)x2_row[b] * nmo + m] = mo64[(size_t)b * nmo + m];
+  // (the table of powers is the same for every wavefunction: built once, since
+  // qmc_set_params rebuilds the tables at every optimisation step)
+  static const std::vector<double> exp2_tab = [] {
+    std::vector<double> t(2048);
+    for (int j = 0; j < 2048; ++j) t[j] = (double)std::exp2((long double)j / 2048.0L);
+    return t;
+  }();
+  // position of AO b's primitives with the AOs in canonical order
+  std::vector<int> prim_val(h.prim_start[nao]);
+  for (const ShellDev& q : shells)
+    for (int k = 0; k < q.n_ao; ++k)
+      for (int p = 0; p < q.n_prim; ++p)
+        prim_val[h.prim_start[q.ao_first + k] + p] =
+            h.prim_start[q.ao_first] + (x2_row[q.ao_first + k] - q.ao_first) * q.n_prim + p;
+  d.log_w0 = ndet == 1 ? std::log(std::fabs(h.det_w[0])) : 0.0;
+
   // ---- determinants: unique excitation records per spin.  The expansion is
   // stored sorted by (rank up, rank down): the determinant stage hands
   // consecutive determinants to the lanes of a warp, and a sorted list keeps
@@ -603,6 +633,7 @@ qmc_status build_tables(qmc_wf* wf) {
     d.nh[s] = ns - h_lo;
     d.nv[s] = p_hi - ns;
   }
+  d.n_col = std::max(1, std::max(d.p_hi[0], d.p_hi[1]));
   d.tab_elems = 2 * (d.nh[0] * d.nv[0] + d.nh[1] * d.nv[1]);
   // per determinant and spin: the table offsets (h_a - h_lo) nv + (p_b - n_s)
   // of its k x k block packed into one word (8 bits each; nh nv <= 8 x 24)
@@ -706,7 +737,10 @@ qmc_status build_tables(qmc_wf* wf) {
       {tc_shells.data(), sizeof(int) * tc_shells.size()}, {det_tab.data(), sizeof(int) * det_tab.size()},
       {mo_x2.data(), sizeof(float) * mo_x2.size()},      {exp_tab.data(), sizeof(float) * exp_tab.size()},
       {mo_oz.data(), sizeof(uint16_t) * mo_oz.size()},  {oz_bnd.data(), sizeof(float) * oz_bnd.size()},
-      {order.data(), sizeof(int) * order.size()},        {mo_x2n.data(), sizeof(float) * mo_x2n.size()}};
+      {order.data(), sizeof(int) * order.size()},        {mo_x2n.data(), sizeof(float) * mo_x2n.size()},
+      {mo64c.data(), sizeof(double) * mo64c.size()},     {nak.data(), sizeof(double) * nak.size()},
+      {exp2_tab.data(), sizeof(double) * exp2_tab.size()}, {x2_row.data(), sizeof(int) * nao},
+      {prim_val.data(), sizeof(int) * prim_val.size()}};
   size_t total = 0;
   for (auto& p : parts) total += align256(p.second);
   void* blob = nullptr;
@@ -748,6 +782,14 @@ qmc_status build_tables(qmc_wf* wf) {
   d.oz_bound = have_bnd ? reinterpret_cast<const float4*>(ptr[17]) : nullptr;
   d.det_orig = reinterpret_cast<const int*>(ptr[18]);
   d.mo_x2n = reinterpret_cast<const float2*>(ptr[19]);
+  d.mo64c = reinterpret_cast<const double*>(ptr[20]);
+  d.nak = reinterpret_cast<const double*>(ptr[21]);
+  d.exp2_tab = reinterpret_cast<const double*>(ptr[22]);
+  d.ao_row = reinterpret_cast<const int*>(ptr[23]);
+  d.prim_val = reinterpret_cast<const int*>(ptr[24]);
+  // one lane per electron (k_small.cu) wherever its closed forms apply: FP64
+  // with or without backflow, and the FP32X2 form with backflow
+  d.small = (general_supported(d) && all_sp && !d.mb_en && !d.n_een && (prec == QMC_FP64 || d.gen_x2)) ? 1 : 0;
   // the SIMT pair kernel serves this wavefunction when the tensor-core stage
   // does not fit, or when the contraction is too small to pay for it (H2 and
   // LiH: n_ao x n_mo of 2 and 72, where k_ao_mo_x2 measured 1.1-2.1x faster at
@@ -895,6 +937,12 @@ static void mark(qmc_wf* wf, int k, cudaStream_t st) {
   if (wf->timing) cudaEventRecord(wf->tev[k], st);
 }
 
+// whether the small-molecule kernels serve this wavefunction (the explicit
+// determinant method keeps its own stage without backflow)
+static bool small_path(const qmc_wf* wf) {
+  return wf->dev.small && (wf->det_method == QMC_DET_TABLE || wf->dev.bf_w != 0.0);
+}
+
 // Local-energy (kinetic) or value-only evaluation of W walkers.
 // Stages: Jastrow + Coulomb, AO + AO->MO contraction, determinants (table
 // method, or explicit per-excitation LU when selected), in order on the
@@ -912,6 +960,15 @@ static qmc_status eval_path(qmc_wf* wf, const double* walkers, int64_t W, int64_
                             int* err_flag, bool kinetic, double* e_loc, double* log_psi, cudaStream_t st,
                             const double* mapped = nullptr, double* stage = nullptr) {
   const WfDev& d = wf->dev;
+  if (kinetic && small_path(wf)) {  // one kernel, one lane per electron
+    mark(wf, 0, st);
+    qmc_status s =
+        launch_status(launch_small_energy(d, mapped ? mapped : walkers, W, ldw, e_loc, log_psi, st), "small energy");
+    if (s) return s;
+    for (int k = 1; k < 6; ++k) mark(wf, k, st);
+    if (wf->timing) wf->timed_once = true;
+    return QMC_OK;
+  }
   if (d.bf_w != 0.0) {  // backflow: one general kernel (Jastrow, orbitals, Eq. nabla_d, E_L)
     mark(wf, 0, st);
     qmc_status s = launch_status(launch_eloc_general(d, walkers, W, ldw, kinetic, e_loc, log_psi, st), "general");
@@ -962,6 +1019,7 @@ static qmc_status eval_path(qmc_wf* wf, const double* walkers, int64_t W, int64_
 // workspace's status word first (a later read tells whether this call's waits
 // gave up).
 static bool has_device_waits(const qmc_wf* wf) {
+  if (wf->dev.bf_w != 0.0) return false;  // backflow runs the general kernels only
   return wf->precision == QMC_MIXED_TF32 || wf->precision == QMC_MIXED_BF16 ||
          (wf->precision == QMC_FP32X2 && (wf->dev.oz || wf->dev.tc_value));
 }
@@ -1132,6 +1190,16 @@ qmc_status sample_call(qmc_wf* wf, double* walkers, int64_t n_walkers, int64_t l
   Workspace ws = carve(wf, base, n_walkers, &err_flag);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   if (reset && (s = reset_status(wf, err_flag, st))) return s;
+  if (small_path(wf)) {  // the whole chain in registers
+    mark(wf, 0, st);
+    s = launch_status(launch_small_chain(wf->dev, walkers, n_walkers, ldw, n_steps, step, seed, first_walker,
+                                         step_offset, log_psi, n_accept, st),
+                      "small chain");
+    if (s) return s;
+    for (int k = 1; k < 6; ++k) mark(wf, k, st);
+    if (wf->timing) wf->timed_once = true;
+    return QMC_OK;
+  }
   s = eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, false, nullptr, ws.lp, st);
   if (s) return s;
   Workspace wp = ws;  // value path on the proposals: walkers = prop, ldw = ldm
@@ -1279,14 +1347,14 @@ qmc_status qmc_set_params(qmc_wf* wf, const double* params) {
 }  // extern "C"
 
 // Preconditions and scratch of the energy-gradient calls: the library-owned
-// workspace, and in the gradient scratch e_loc [W], stats [4] and the block
-// partial sums (rows x blocks, rows up to max(n_param, 9 n_atom)).
+// workspace, and in the gradient scratch e_loc [W], the statistics
+// (mean_var_doubles) and the block partial sums (rows x blocks, rows up to max(n_param, 9 n_atom)).
 // The energy-gradient path of a wavefunction: the general kernels (one
 // determinant, <= 8 electrons, <= 4 per spin; gradient and forces) or the
 // multi-determinant kernels (no backflow; gradient only).
 static qmc_status grad_setup(qmc_wf* wf, const double* walkers, int64_t n_walkers, int64_t ldw, bool want_grad,
                              int64_t* n_param, Workspace* ws, int** err_flag, double** e_loc, double** stats,
-                             double** partial, bool* md) {
+                             double** partial, bool* md, bool* small) {
   if (!wf) return fail(QMC_ERR_ARG, "null wavefunction");
   if (n_walkers < 1 || ldw < n_walkers) return fail(QMC_ERR_ARG, "need n_walkers >= 1 and ldw >= n_walkers");
   if (!walkers) return fail(QMC_ERR_ARG, "null walkers");
@@ -1309,9 +1377,13 @@ static qmc_status grad_setup(qmc_wf* wf, const double* walkers, int64_t n_walker
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  const size_t part = *md ? md_grad_scratch_bytes(wf->dev, ws->ldm, (int)*n_param, n_sm)
-                          : sizeof(double) * nb * std::max<int64_t>(*n_param, 9 * wf->dev.n_atom);
-  const size_t need = align256(sizeof(double) * n_walkers) + align256(sizeof(double) * 4) + align256(part);
+  const int n_prim = wf->spec.prim_start[wf->dev.n_ao];
+  *small = !*md && small_path(wf) && small_grad_supported(wf->dev, n_prim);
+  const size_t part = *md      ? md_grad_scratch_bytes(wf->dev, ws->ldm, (int)*n_param, n_sm)
+                      : *small ? small_grad_scratch_bytes(wf->dev, n_walkers, n_prim)
+                               : sizeof(double) * nb * std::max<int64_t>(*n_param, 9 * wf->dev.n_atom);
+  const size_t sb = align256(sizeof(double) * mean_var_doubles(n_walkers));
+  const size_t need = align256(sizeof(double) * n_walkers) + sb + align256(part);
   if (wf->gws_bytes < need) {
     if (wf->gws) cudaFree(wf->gws);
     wf->gws = nullptr;
@@ -1326,7 +1398,7 @@ static qmc_status grad_setup(qmc_wf* wf, const double* walkers, int64_t n_walker
   char* p = static_cast<char*>(wf->gws);
   *e_loc = reinterpret_cast<double*>(p);
   *stats = reinterpret_cast<double*>(p + align256(sizeof(double) * n_walkers));
-  *partial = reinterpret_cast<double*>(p + align256(sizeof(double) * n_walkers) + align256(sizeof(double) * 4));
+  *partial = reinterpret_cast<double*>(p + align256(sizeof(double) * n_walkers) + sb);
   return QMC_OK;
 }
 
@@ -1343,17 +1415,29 @@ qmc_status qmc_energy_grad(qmc_wf* wf, const double* walkers, int64_t n_walkers,
   Workspace ws;
   int* err_flag;
   double *e_loc, *stats, *partial;
-  bool md = false;
+  bool md = false, small = false;
   qmc_status s = grad_setup(wf, walkers, n_walkers, ldw, grad != nullptr, &n_param, &ws, &err_flag, &e_loc, &stats,
-                            &partial, &md);
+                            &partial, &md, &small);
   if (s) return s;
   if (md && forces)
     return fail(QMC_ERR_UNSUPPORTED,
                 "forces need one determinant with <= 8 electrons and no many-body Jastrow (pass forces = NULL)");
-  s = eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
+  const int n_prim = wf->spec.prim_start[wf->dev.n_ao];
+  small = small && (grad || forces);  // statistics alone: the energy kernel
+  s = small ? launch_status(launch_small_grad(wf->dev, walkers, n_walkers, ldw, wf->dev.ao_prim, n_prim, e_loc,
+                                              partial, st),
+                            "energies and gradient sums")
+            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
   if (s) return s;
   s = launch_status(launch_mean_var(e_loc, n_walkers, stats, st), "mean/variance");
   if (s) return s;
+  if (small) {
+    s = launch_status(launch_small_assemble(wf->dev, n_walkers, n_prim, (int)n_param, stats, 0, partial, grad, forces,
+                                            st),
+                      "gradient assembly");
+    if (s) return s;
+    grad = forces = nullptr;  // done
+  }
   if (grad && md) {
     s = launch_status(launch_md_grad(wf->dev, walkers, n_walkers, ldw, ws, e_loc, stats, wf->spec.prim_start[wf->dev.n_ao],
                                      (int)n_param, partial, grad, st),
@@ -1392,14 +1476,22 @@ qmc_status qmc_energy_grad_sums(qmc_wf* wf, const double* walkers, int64_t n_wal
   Workspace ws;
   int* err_flag;
   double *e_loc, *stats, *partial;
-  bool md = false;
+  bool md = false, small = false;
   qmc_status s =
-      grad_setup(wf, walkers, n_walkers, ldw, true, &n_param, &ws, &err_flag, &e_loc, &stats, &partial, &md);
+      grad_setup(wf, walkers, n_walkers, ldw, true, &n_param, &ws, &err_flag, &e_loc, &stats, &partial, &md, &small);
   if (s) return s;
-  s = eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
+  const int n_prim = wf->spec.prim_start[wf->dev.n_ao];
+  s = small ? launch_status(launch_small_grad(wf->dev, walkers, n_walkers, ldw, wf->dev.ao_prim, n_prim, e_loc,
+                                              partial, st),
+                            "energies and gradient sums")
+            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
   if (s) return s;
   s = launch_status(launch_energy_sums(e_loc, n_walkers, sums, st), "energy sums");
   if (s) return s;
+  if (small)
+    return launch_status(launch_small_assemble(wf->dev, n_walkers, n_prim, (int)n_param, stats, 1, partial, sums + 3,
+                                               sums + 3 + 2 * n_param, st),
+                         "gradient sums");
   if (md) {  // gradient sums; the force blocks are NaN (forces need path (a))
     for (int weight = 1; weight <= 2 && !s; ++weight)
       s = launch_status(launch_md_grad(wf->dev, walkers, n_walkers, ldw, ws, e_loc, stats,

@@ -13,7 +13,7 @@ namespace qmc {
 template <typename T, int NMO, int NCH>
 __global__ void __launch_bounds__(128) k_ao_mo_simt(WfDev wf, const double* __restrict__ walkers, int64_t W,
                                                     int64_t ldw, const T* __restrict__ gradJ,
-                                                    double* __restrict__ mo_out, int64_t ldm) {
+                                                    double* __restrict__ mo_out, int nmp, int64_t ldm) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   ShellDev* sh_s = reinterpret_cast<ShellDev*>(smem_raw);
   int* pow_s = reinterpret_cast<int*>(sh_s + wf.n_shell);
@@ -79,12 +79,12 @@ __global__ void __launch_bounds__(128) k_ao_mo_simt(WfDev wf, const double* __re
       }
     }
   }
-  // walker-fastest FP64 MO layout [N][NCH][NMO][ldm] (FP32 results widened exactly)
-  double* dst = mo_out + (size_t)i * NCH * NMO * ldm + w;
+  // walker-fastest FP64 MO layout [N][NCH][nmp][ldm] (FP32 results widened exactly)
+  double* dst = mo_out + (size_t)i * NCH * nmp * ldm + w;
 #pragma unroll
   for (int m = 0; m < NMO; ++m) {
     dst[(size_t)m * ldm] = widen(acc0[m]);
-    if (NCH == 2) dst[(size_t)(NMO + m) * ldm] = widen(acc1[m]);
+    if (NCH == 2) dst[(size_t)(nmp + m) * ldm] = widen(acc1[m]);
   }
 }
 
@@ -95,22 +95,26 @@ static cudaError_t launch_t(const WfDev& wf, const double* walkers, int64_t W, i
   const T* gj = static_cast<const T*>(ws.gradJ);
   double* mo = ws.mo;
 #define QMC_AOMO(NM)                                                                                        \
-  if (wf.n_mo <= NM) {                                                                                      \
+  if (wf.n_col <= NM) {                                                                                     \
     const size_t smem = round_up(sizeof(ShellDev) * wf.n_shell + sizeof(int) * wf.n_ao, 16) +              \
                         sizeof(T) * wf.n_ao * NM;                                                           \
     if (nch == 2) {                                                                                         \
       auto kern = k_ao_mo_simt<T, NM, 2>;                                                                   \
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                   \
-      kern<<<grid, block, smem, st>>>(wf, walkers, W, ldw, gj, mo, ws.ldm);                                 \
+      kern<<<grid, block, smem, st>>>(wf, walkers, W, ldw, gj, mo, ws.nmp, ws.ldm);                         \
     } else {                                                                                                \
       auto kern = k_ao_mo_simt<T, NM, 1>;                                                                   \
       cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);                   \
-      kern<<<grid, block, smem, st>>>(wf, walkers, W, ldw, gj, mo, ws.ldm);                                 \
+      kern<<<grid, block, smem, st>>>(wf, walkers, W, ldw, gj, mo, ws.nmp, ws.ldm);                         \
     }                                                                                                       \
     return cudaGetLastError();                                                                              \
   }
   if (ws.nmp != mo_row_pad(wf.n_mo, false)) return cudaErrorInvalidValue;
+  // brackets of the columns that the determinant stage reads
+  QMC_AOMO(2)
+  QMC_AOMO(4)
   QMC_AOMO(8)
+  QMC_AOMO(14)
   QMC_AOMO(16)
   QMC_AOMO(32)
 #undef QMC_AOMO

@@ -53,30 +53,69 @@ __global__ void __launch_bounds__(128) k_logpsi_general(const __grid_constant__ 
   log_psi[w] = logpsi_walker<NE, NO, PAIRS>(wf, g, r);
 }
 
-// Sum of W values in a fixed order: [0] mean, [1] mean square deviation.
-__global__ void k_mean_var(const double* __restrict__ x, int64_t W, double* __restrict__ stats) {
+// Mean and mean square deviation of W values in a fixed order.  Blocks of
+// kMvChunk values form their own mean and sum of squared deviations (values
+// in registers, read once); one block then combines them,
+//   mean = sum n_i m_i / W,  var = sum (M2_i + n_i (m_i - mean)^2) / W.
+// (One block over all values was a serial chain of loads: 73 us at 65,536.)
+constexpr int kMvChunk = 2048;
+
+__device__ double block_sum256(double v, double* red) {
+  __syncthreads();
+  red[threadIdx.x] = v;
+  __syncthreads();
+  for (int o = 128; o > 0; o >>= 1) {
+    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
+    __syncthreads();
+  }
+  return red[0];
+}
+
+__global__ void __launch_bounds__(256) k_mean_var_part(const double* __restrict__ x, int64_t W,
+                                                       double* __restrict__ part) {
   __shared__ double red[256];
-  double s = 0.0;
-  for (int64_t k = threadIdx.x; k < W; k += blockDim.x) s += x[k];
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  constexpr int kPer = kMvChunk / 256;
+  const int64_t k0 = (int64_t)blockIdx.x * kMvChunk;
+  const int64_t left = W - k0;
+  const double n = (double)(left < kMvChunk ? left : kMvChunk);
+  double v[kPer], s = 0.0;
+#pragma unroll
+  for (int q = 0; q < kPer; ++q) {
+    const int64_t k = k0 + q * 256 + threadIdx.x;
+    v[q] = k < W ? x[k] : 0.0;
+    s += v[q];
   }
-  const double mean = red[0] / (double)W;
-  __syncthreads();
+  const double mean = block_sum256(s, red) / n;
   s = 0.0;
-  for (int64_t k = threadIdx.x; k < W; k += blockDim.x) s += (x[k] - mean) * (x[k] - mean);
-  red[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if ((int)threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+#pragma unroll
+  for (int q = 0; q < kPer; ++q)
+    if (k0 + q * 256 + threadIdx.x < W) s = fma(v[q] - mean, v[q] - mean, s);
+  const double m2 = block_sum256(s, red);
+  if (threadIdx.x == 0) {
+    part[2 * blockIdx.x] = mean;
+    part[2 * blockIdx.x + 1] = m2;
   }
+}
+
+__global__ void __launch_bounds__(256) k_mean_var_all(const double* __restrict__ part, int n_part, int64_t W,
+                                                      double* __restrict__ stats) {
+  __shared__ double red[256];
+  auto count = [&](int c) {
+    const int64_t left = W - (int64_t)c * kMvChunk;
+    return (double)(left < kMvChunk ? left : kMvChunk);
+  };
+  double s = 0.0;
+  for (int c = threadIdx.x; c < n_part; c += 256) s = fma(count(c), part[2 * c], s);
+  const double mean = block_sum256(s, red) / (double)W;
+  s = 0.0;
+  for (int c = threadIdx.x; c < n_part; c += 256) {
+    const double d = part[2 * c] - mean;
+    s += fma(count(c) * d, d, part[2 * c + 1]);
+  }
+  s = block_sum256(s, red);
   if (threadIdx.x == 0) {
     stats[0] = mean;
-    stats[1] = red[0] / (double)W;
+    stats[1] = s / (double)W;
   }
 }
 
@@ -169,8 +208,14 @@ cudaError_t launch_mean_var_finite(const double* x, int64_t W, double* stats, cu
   return cudaGetLastError();
 }
 
+size_t mean_var_doubles(int64_t W) { return 4 + 2 * (size_t)((W + kMvChunk - 1) / kMvChunk); }
+
 cudaError_t launch_mean_var(const double* x, int64_t W, double* stats, cudaStream_t st) {
-  k_mean_var<<<1, 256, 0, st>>>(x, W, stats);
+  const int n = (int)((W + kMvChunk - 1) / kMvChunk);
+  k_mean_var_part<<<n, 256, 0, st>>>(x, W, stats + 4);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_mean_var_all<<<1, 256, 0, st>>>(stats + 4, n, W, stats);
   return cudaGetLastError();
 }
 

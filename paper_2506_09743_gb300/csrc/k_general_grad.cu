@@ -183,17 +183,24 @@ __global__ void __launch_bounds__(128) k_grad_logpsi(WfDev wf, const double* __r
   for (int k = tid; k < n_param; k += T) partial[(size_t)k * gridDim.x + blockIdx.x] = acc[(size_t)k * T];
 }
 
-// Row sums of partial[n_rows][n_cols] in column order (deterministic).
-__global__ void k_row_sums(const double* __restrict__ partial, int n_rows, int n_cols, double* __restrict__ out) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+// Row sums of partial[n_rows][n_cols] in a fixed order (deterministic): one
+// warp per row, lane l adds columns l, l + 32, ... in order, then a shuffle
+// tree.  (One thread per row read its row uncoalesced: 119 us for 1,008 rows
+// of 1,216 columns.)
+__global__ void __launch_bounds__(128) k_row_sums(const double* __restrict__ partial, int n_rows, int n_cols,
+                                                  double* __restrict__ out) {
+  const int k = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (k >= n_rows) return;
   double s = 0.0;
-  for (int c = 0; c < n_cols; ++c) s += partial[(size_t)k * n_cols + c];
-  out[k] = s;
+#pragma unroll 4
+  for (int c = lane; c < n_cols; c += 32) s += partial[(size_t)k * n_cols + c];
+#pragma unroll
+  for (int o = 16; o >= 1; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (lane == 0) out[k] = s;
 }
 
 cudaError_t launch_row_sums(const double* partial, int n_rows, int n_cols, double* out, cudaStream_t st) {
-  k_row_sums<<<(n_rows + 127) / 128, 128, 0, st>>>(partial, n_rows, n_cols, out);
+  k_row_sums<<<(n_rows + 3) / 4, 128, 0, st>>>(partial, n_rows, n_cols, out);
   return cudaGetLastError();
 }
 
@@ -208,8 +215,7 @@ cudaError_t launch_forces(const WfDev& wf, const double* walkers, int64_t W, int
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int rows = (raw ? 9 : 3) * wf.n_atom;
-  k_row_sums<<<(rows + 127) / 128, 128, 0, st>>>(partial, rows, grid.x, forces);
-  return cudaGetLastError();
+  return launch_row_sums(partial, rows, (int)grid.x, forces, st);
 }
 
 size_t grad_smem_bytes(const WfDev& wf, int n_param) { return gen_table_bytes(wf) + sizeof(double) * 128 * n_param; }
@@ -225,8 +231,7 @@ cudaError_t launch_grad(const WfDev& wf, const double* walkers, int64_t W, int64
                                                                    prim_start, n_param, partial, weight)));
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_row_sums<<<(n_param + 127) / 128, 128, 0, st>>>(partial, n_param, grid.x, grad);
-  return cudaGetLastError();
+  return launch_row_sums(partial, n_param, (int)grid.x, grad, st);
 }
 
 // M, sum E_L and sum E_L^2 of a batch in a fixed order (one block)

@@ -75,6 +75,7 @@ struct WfDev {
   int h_lo[2];    // smallest hole index per spin (n_s if none)
   int p_hi[2];    // one past the largest particle index per spin (n_s if none)
   int nh[2], nv[2];  // table extents: holes n_s - h_lo, virtuals p_hi - n_s
+  int n_col;      // orbital columns the determinant stage reads (largest p_hi): the SIMT AO stages form no others
   int tab_elems;  // doubles of excitation tables per walker
   double w0_par, w0_anti, jb, bf_w, vnn;
   float w0p_f, w0a_f, jb_f;  // FP32 copies for the FP32 kernels
@@ -119,6 +120,18 @@ struct WfDev {
   // core-matrix layout [n_mo_pad=16][k_pad], 32-bit words
   const uint32_t* mo_tc_hi;
   const uint32_t* mo_tc_lo;
+  // small-molecule path (small_eval.cuh): 1 when it serves this wavefunction
+  // (one determinant, <= 8 electrons, <= 4 per spin, complete s and p shells);
+  // MO table rows in canonical shell order, -2048 alpha / ln 2 per shell and
+  // primitive, 2^(j/2048), whether any shell is a Slater function, log|d_0|
+  int small;
+  int any_sto;
+  double log_w0;
+  const double* mo64c;     // [n_ao][n_mo]
+  const double* nak;       // [n_shell][QMC_MAX_PRIM]
+  const double* exp2_tab;  // [2048]
+  const int* ao_row;       // [n_ao] canonical row of each AO
+  const int* prim_val;     // [n_prim] position of each primitive's exponent with the AOs in canonical order
   const double* ao_ang;  // [n_ao] angular normalisation factors (folded into mo64)
   const int* ao_prim;    // [n_ao + 1] first input primitive of each AO (gradient layout)
   // tensor-core AO stage: AO b sits in column ao_col[b] of the K dimension,
@@ -283,6 +296,24 @@ cudaError_t launch_md_grad(const WfDev& wf, const double* walkers, int64_t W, in
                            double* grad, cudaStream_t st, int weight = 0);
 cudaError_t launch_eloc_general(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, bool kinetic,
                                 double* e_loc, double* log_psi, cudaStream_t st);
+// small-molecule path: E_L and log|Psi|; n_steps Metropolis steps in one launch
+cudaError_t launch_small_energy(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, double* e_loc,
+                                double* log_psi, cudaStream_t st);
+cudaError_t launch_small_chain(const WfDev& wf, double* walkers, int64_t W, int64_t ldw, int32_t n_steps, double step,
+                               uint64_t seed, uint64_t first_walker, uint64_t step_offset, double* log_psi,
+                               int64_t* n_accept, cudaStream_t st);
+// the same path's gradient and forces: per-warp sums (and e_loc) first, then,
+// once stats holds the mean energy, their assembly (mode 0: the estimators of
+// Eqs. nabla_loss and force; mode 1: the raw sums of a sharded batch)
+bool small_grad_supported(const WfDev& wf, int n_prim);
+size_t small_grad_scratch_bytes(const WfDev& wf, int64_t W, int n_prim);
+cudaError_t launch_small_grad(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, const int* prim_start,
+                              int n_prim, double* e_loc, double* scratch, cudaStream_t st);
+cudaError_t launch_small_assemble(const WfDev& wf, int64_t W, int n_prim, int n_param, const double* stats, int mode,
+                                  double* scratch, double* grad, double* forces, cudaStream_t st);
+// stats[0..1] = mean, mean square deviation; stats holds mean_var_doubles(W)
+// doubles (block results behind the first two)
+size_t mean_var_doubles(int64_t W);
 cudaError_t launch_mean_var(const double* x, int64_t W, double* stats, cudaStream_t st);
 // mean and variance of the finite values; stats[2] = number of non-finite values
 cudaError_t launch_mean_var_finite(const double* x, int64_t W, double* stats, cudaStream_t st);

@@ -419,6 +419,13 @@ struct KahanF {
     c = (t - s) - y;
     s = t;
   }
+  // add(a b) with the product unrounded
+  __device__ __forceinline__ void add_product(float a, float b) {
+    const float y = __fmaf_rn(a, b, -c);
+    const float t = s + y;
+    c = (t - s) - y;
+    s = t;
+  }
   __device__ __forceinline__ double value() const { return (double)s - (double)c; }
 };
 
@@ -588,6 +595,265 @@ __global__ void __launch_bounds__(128) k_jastrow_f32(WfDev wf, const double* __r
   jscal[w] = J.value();
   jscal[ldm + w] = VX2 ? lap.value() + lapd : lap.value();
   jscal[2 * ldm + w] = (VX2 ? widen(vx) + V.value() + Vd : V.value()) + wf.vnn;
+}
+
+// ---- FP32X2 Jastrow stage, walkers over lanes and a walker's pairs over warps.
+//
+// One thread per walker (k_jastrow_f32) unrolls every pair: at 14 electrons
+// its body outgrows the instruction cache (issue slots 31% busy, 268 us per
+// 262,144 CO walkers) and a small batch has too few threads (38 us for 4,099
+// walkers).  Here a block holds 32 walkers, one per lane, and
+//   1. stages their positions (float pairs) in shared memory;
+//   2. deals the pairs to its warps in contiguous ranges: geometry, the factors
+//      of the J, Laplacian and Coulomb terms and u'/r go to shared memory, and
+//      the electron-nucleus potential is summed per warp in pairs;
+//   3. sums: a warp per electron gathers grad_i J over its partners in ascending
+//      order, and three warps run the compensated sums of J, V and the
+//      Laplacian over the pairs in order.
+// The sums keep k_jastrow_f32's order and operations, so J, grad J, the kinetic
+// scalar and the electron-electron potential are the same bit for bit (the
+// electron-nucleus pairs are added in another order, 2^-47 of V).  The FP32
+// forms and value-only calls stay with k_jastrow_f32: there the compiler joins
+// products and sums of the J chain into FMAs pair by pair in its own way, and
+// log|Psi| would move by 3e-9.
+constexpr int kJwThreads = 512;
+constexpr int kJwWarps = kJwThreads / 32;
+constexpr int kJwMinElec = 6;  // at most this many electrons: one thread per walker
+// floats per lane of an electron's record (hi, lo of x, y, z) and of a pair's:
+// J factors (2), Laplacian, 1/r, u'/r, r_i - r_j (3).  A record's fields are 32
+// floats apart, so one address and immediate offsets reach all of them.
+constexpr int kJwPos = 6, kJwPair = 8;
+
+__host__ __device__ inline int jw_rows(int n) {
+  return kJwPos * n + kJwPair * (n * (n - 1) / 2) + 3 * n + 2 * kJwWarps;
+}
+
+template <bool MB>
+__global__ void __launch_bounds__(kJwThreads) k_jastrow_wide(const __grid_constant__ WfDev wf, const double* walkers,
+                                                             int64_t W, int64_t ldw, double* copy,
+                                                             float* __restrict__ gradJ, double* __restrict__ jscal,
+                                                             int64_t ldm, float b, float w0p, float w0a) {
+  extern __shared__ float sm[];
+  __shared__ int any_close[32];
+  __shared__ uchar2 pair_s[kEenMaxPairs];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int n = wf.n_elec, np = n * (n - 1) / 2;
+  const int64_t w = (int64_t)blockIdx.x * 32 + lane;
+  const bool live = w < W;
+  const int64_t wc = live ? w : W - 1;
+  float* pos = sm + lane;                             // [n][6][32]
+  float* term = pos + kJwPos * n * 32;                // [np][8][32]
+  float* grad = term + kJwPair * np * 32;             // [3n][32]
+  float* enp = grad + 3 * n * 32;                     // [kJwWarps][2][32]
+  for (int k = warp; k < 3 * n; k += kJwWarps) {
+    const double v = walkers[(int64_t)k * ldw + wc];
+    if (copy && live) copy[(int64_t)k * ldw + w] = v;
+    const int i = k / 3;
+    float* p = pos + (kJwPos * i + (k - 3 * i)) * 32;
+    split_f64(v, p[0], p[3 * 32]);
+  }
+  if (threadIdx.x < n) {
+    const int i = threadIdx.x;
+    for (int j = i + 1; j < n; ++j)
+      pair_s[i * n - i * (i + 1) / 2 + (j - i - 1)] = make_uchar2((unsigned char)i, (unsigned char)j);
+  }
+  if (threadIdx.x < 32) any_close[threadIdx.x] = 0;
+  __syncthreads();
+  // ---- pairs: ranges (i, j), (i, j + 1), ...
+  {
+    const int k1 = (np * (warp + 1)) / kJwWarps;
+    int k = (np * warp) / kJwWarps;
+    float* t = term + kJwPair * 32 * k;
+    while (k < k1) {
+      const int i = pair_s[k].x;
+      int j = pair_s[k].y;
+      const float* pi = pos + kJwPos * 32 * i;
+      const float xh = pi[0], yh = pi[32], zh = pi[64], xl = pi[96], yl = pi[128], zl = pi[160];
+      const float* pj = pos + kJwPos * 32 * j;
+      for (; j < n && k < k1; ++j, ++k, pj += kJwPos * 32, t += kJwPair * 32) {
+        const float dx = (xh - pj[0]) + (xl - pj[96]);
+        const float dy = (yh - pj[32]) + (yl - pj[128]);
+        const float dz = (zh - pj[64]) + (zl - pj[160]);
+        const float d2 = __fmaf_rn(dz, dz, __fmaf_rn(dy, dy, __fmul_rn(dx, dx)));
+        const float inv = rsqrtf(d2);
+        const float dist = d2 * inv;
+        const float w0 = ((i < wf.n_up) == (j < wf.n_up)) ? w0p : w0a;
+        const float rden = __frcp_rn(1.0f + b * dist);
+        const float u1 = w0 * rden * rden;
+        const bool close = d2 < 1e-4f;
+        if (close) any_close[lane] = 1;
+        const float e = fmaf(-d2 * inv, inv, 1.0f);
+        t[0] = w0 * dist;
+        t[32] = rden;
+        t[64] = close ? 0.0f : 2.0f * (-2.0f * b * u1 * rden + 2.0f * u1 * inv);
+        t[96] = close ? 0.0f : fmaf(0.5f * inv, e, inv);
+        t[128] = u1 * inv;
+        t[160] = dx;
+        t[192] = dy;
+        t[224] = dz;
+      }
+    }
+  }
+  const double* src = copy ? copy : walkers;  // written above by this block where copied
+  {
+    // electron-nucleus potential in pairs (r_i - R_a from the FP64 coordinates)
+    f32x2 vx(0.f, 0.f);
+    const int m = n * wf.n_atom;
+    for (int k = kJwWarps - 1 - warp; k < m; k += kJwWarps) {
+      const int a = k / n, i = k - a * n;
+      float zh, zl;
+      split_f64(wf.atom_z[a], zh, zl);
+      f32x2 dv[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) dv[d] = diff_x2(src[(int64_t)(3 * i + d) * ldw + wc], wf.atom_xyz[a][d]);
+      vx = vx - inv_dist_x2(dv[0], dv[1], dv[2]) * f32x2(zh, zl);
+    }
+    enp[(2 * warp) * 32] = vx.hi;
+    enp[(2 * warp + 1) * 32] = vx.lo;
+  }
+  __syncthreads();
+  // ---- sums: electrons over the first warps, J, V and the Laplacian on the last three
+  auto en_disp = [&](int i, int a, float* v) {
+    for (int d = 0; d < 3; ++d) {
+      float ah, al;
+      split_f64(wf.atom_xyz[a][d], ah, al);
+      v[d] = (pos[(kJwPos * i + d) * 32] - ah) + (pos[(kJwPos * i + 3 + d) * 32] - al);
+    }
+  };
+  const float w0e = wf.jen_f[0], w1e = wf.jen_f[1], w2e = wf.jen_f[2];
+  KahanF lap;
+  double lapd = 0.0;
+  if (warp < kJwWarps - 3) {
+    for (int e = warp; e < n; e += kJwWarps - 3) {
+      float gx = 0.f, gy = 0.f, gz = 0.f;
+      // partners o < e: pair (o, e), n - o - 2 records apart; this electron is its second
+      const float* t = term + kJwPair * 32 * (e - 1);
+      for (int o = 0; o < e; ++o) {
+        const float s = -t[128];
+        gx += s * t[160];
+        gy += s * t[192];
+        gz += s * t[224];
+        t += kJwPair * 32 * (n - o - 2);
+      }
+      // partners o > e: consecutive records
+      t = term + kJwPair * 32 * (e * n - e * (e + 1) / 2);
+#pragma unroll 4
+      for (int o = e + 1; o < n; ++o, t += kJwPair * 32) {
+        const float s = t[128];
+        gx += s * t[160];
+        gy += s * t[192];
+        gz += s * t[224];
+      }
+      if (MB && wf.mb_en) {
+        for (int a = 0; a < wf.n_atom; ++a) {
+          float v[3];
+          en_disp(e, a, v);
+          const float r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+          const float ir = 1.0f / sqrtf(r2), r = r2 * ir;
+          const float id = 1.0f / (1.0f + w2e * r);
+          const float k1 = (w0e + 2.0f * w1e * r + w1e * w2e * r * r) * id * id;
+          const float s = k1 * ir;
+          gx += s * v[0];
+          gy += s * v[1];
+          gz += s * v[2];
+        }
+      }
+      grad[(3 * e) * 32] = gx;
+      grad[(3 * e + 1) * 32] = gy;
+      grad[(3 * e + 2) * 32] = gz;
+      if (live) {
+        gradJ[(int64_t)(3 * e) * ldm + w] = gx;
+        gradJ[(int64_t)(3 * e + 1) * ldm + w] = gy;
+        gradJ[(int64_t)(3 * e + 2) * ldm + w] = gz;
+      }
+    }
+  } else if (warp == kJwWarps - 3) {  // J
+    KahanF J;
+    const float* t = term;
+#pragma unroll 8
+    for (int k = 0; k < np; ++k, t += kJwPair * 32) J.add_product(t[0], t[32]);
+    if (MB && wf.mb_en)
+      for (int a = 0; a < wf.n_atom; ++a)
+        for (int i = 0; i < n; ++i) {
+          float v[3];
+          en_disp(i, a, v);
+          const float r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+          const float ir = 1.0f / sqrtf(r2), r = r2 * ir;
+          const float id = 1.0f / (1.0f + w2e * r);
+          J.add((w0e * r + w1e * r * r) * id);
+        }
+    if (live) jscal[w] = J.value();
+  } else if (warp == kJwWarps - 2) {  // V
+    KahanF V;
+    const float* t = term + 96;
+#pragma unroll 8
+    for (int k = 0; k < np; ++k, t += kJwPair * 32) V.add(t[0]);
+    double Vd = 0.0;  // close pairs in FP64
+    if (any_close[lane]) {
+      for (int k = 0; k < np; ++k) {
+        const float* p = term + kJwPair * 32 * k + 160;
+        if (!(__fmaf_rn(p[64], p[64], __fmaf_rn(p[32], p[32], __fmul_rn(p[0], p[0]))) < 1e-4f)) continue;
+        const int i = pair_s[k].x, j = pair_s[k].y;
+        double dd2 = 0.0;
+        for (int d = 0; d < 3; ++d) {
+          const double v = src[(int64_t)(3 * i + d) * ldw + wc] - src[(int64_t)(3 * j + d) * ldw + wc];
+          dd2 += v * v;
+        }
+        Vd += 1.0 / sqrt(dd2);
+      }
+    }
+    f32x2 vx(0.f, 0.f);
+    for (int q = 0; q < kJwWarps; ++q) vx = vx + f32x2(enp[(2 * q) * 32], enp[(2 * q + 1) * 32]);
+    if (live) jscal[2 * ldm + w] = widen(vx) + V.value() + Vd + wf.vnn;
+  } else {  // Laplacian of J over the pairs
+    const float* t = term + 64;
+#pragma unroll 8
+    for (int k = 0; k < np; ++k, t += kJwPair * 32) lap.add(t[0]);
+    if (any_close[lane]) {
+      for (int k = 0; k < np; ++k) {
+        const float* p = term + kJwPair * 32 * k + 160;
+        if (!(__fmaf_rn(p[64], p[64], __fmaf_rn(p[32], p[32], __fmul_rn(p[0], p[0]))) < 1e-4f)) continue;
+        const int i = pair_s[k].x, j = pair_s[k].y;
+        double dd2 = 0.0;
+        for (int d = 0; d < 3; ++d) {
+          const double v = src[(int64_t)(3 * i + d) * ldw + wc] - src[(int64_t)(3 * j + d) * ldw + wc];
+          dd2 += v * v;
+        }
+        const double invd = 1.0 / sqrt(dd2), distd = dd2 * invd;
+        const double w0d = ((i < wf.n_up) == (j < wf.n_up)) ? wf.w0_par : wf.w0_anti;
+        const double rdd = 1.0 / (1.0 + wf.jb * distd), u1d = w0d * rdd * rdd;
+        lapd += 2.0 * (-2.0 * wf.jb * u1d * rdd + 2.0 * u1d * invd);
+      }
+    }
+    if (MB && wf.mb_en)
+      for (int a = 0; a < wf.n_atom; ++a)
+        for (int i = 0; i < n; ++i) {
+          float v[3];
+          en_disp(i, a, v);
+          const float r2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
+          const float ir = 1.0f / sqrtf(r2), r = r2 * ir;
+          const float id = 1.0f / (1.0f + w2e * r);
+          const float k1 = (w0e + 2.0f * w1e * r + w1e * w2e * r * r) * id * id;
+          const float k2 = 2.0f * (w1e - w0e * w2e) * id * id * id;
+          lap.add(k2 + 2.0f * k1 * ir);
+        }
+  }
+  __syncthreads();
+  if (warp == kJwWarps - 1) {
+#pragma unroll 6
+    for (int k = 0; k < 3 * n; ++k) lap.add_product(grad[k * 32], grad[k * 32]);
+    if (live) jscal[ldm + w] = lap.value() + lapd;
+  }
+}
+
+template <bool MB>
+cudaError_t launch_jastrow_wide(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, double* copy,
+                                const Workspace& ws, cudaStream_t st) {
+  const size_t smem = (size_t)jw_rows(wf.n_elec) * 32 * sizeof(float);
+  cudaFuncSetAttribute(k_jastrow_wide<MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_jastrow_wide<MB><<<(unsigned)((W + 31) / 32), kJwThreads, smem, st>>>(
+      wf, walkers, W, ldw, copy, static_cast<float*>(ws.gradJ), ws.jscal, ws.ldm, wf.jb_f, wf.w0p_f, wf.w0a_f);
+  return cudaGetLastError();
 }
 
 // Launch one kernel instance; NM is the electron-count bracket.  If copy is

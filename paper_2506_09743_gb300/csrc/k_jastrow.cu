@@ -17,6 +17,7 @@ cudaError_t launch_jastrow(const WfDev& wf, int prec, const double* walkers, int
   // occupancy with them (14 electrons at NMAX 14: 155 registers, 12 warps/SM;
   // at NMAX 16: 179 registers, 8 warps/SM)
   const int n = wf.n_elec;
+  if (prec == QMC_FP32X2 && derivs && n > kJwMinElec) return launch_jastrow_wide<false>(wf, walkers, W, ldw, copy, ws, st);
   if (n <= 2) return launch_jastrow_nm<2, false>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
   if (n <= 4) return launch_jastrow_nm<4, false>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
   if (n <= 6) return launch_jastrow_nm<6, false>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);

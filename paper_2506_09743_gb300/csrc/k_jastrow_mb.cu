@@ -12,7 +12,8 @@ cudaError_t launch_jastrow_mb(const WfDev& wf, int prec, const double* walkers, 
                               double* copy, const Workspace& ws, bool derivs, cudaStream_t st) {
   const int n = wf.n_elec;
   cudaError_t e;
-  if (n <= 2) e = launch_jastrow_nm<2, true>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
+  if (prec == QMC_FP32X2 && derivs && n > kJwMinElec) e = launch_jastrow_wide<true>(wf, walkers, W, ldw, copy, ws, st);
+  else if (n <= 2) e = launch_jastrow_nm<2, true>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
   else if (n <= 4) e = launch_jastrow_nm<4, true>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
   else if (n <= 8) e = launch_jastrow_nm<8, true>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);
   else if (n <= 16) e = launch_jastrow_nm<16, true>(wf, prec, walkers, W, ldw, copy, ws, derivs, st);

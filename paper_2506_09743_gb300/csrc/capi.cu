@@ -958,7 +958,7 @@ static bool small_path(const qmc_wf* wf) {
 // the device copy (the upload overlaps the Jastrow stage's arithmetic).
 static qmc_status eval_path(qmc_wf* wf, const double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
                             int* err_flag, bool kinetic, double* e_loc, double* log_psi, cudaStream_t st,
-                            const double* mapped = nullptr, double* stage = nullptr) {
+                            const double* mapped = nullptr, double* stage = nullptr, bool averaged = false) {
   const WfDev& d = wf->dev;
   if (kinetic && small_path(wf)) {  // one kernel, one lane per electron
     mark(wf, 0, st);
@@ -997,7 +997,8 @@ static qmc_status eval_path(qmc_wf* wf, const double* walkers, int64_t W, int64_
                     : tc        ? launch_ao_mo_tc(d, wf->precision, walkers, W, ldw, v, nch, err_flag, wf->err_wf, st)
                     : x2 && d.oz ? launch_ao_mo_oz(d, walkers, W, ldw, v, nch, err_flag, wf->err_wf, st)
                     : x2         ? launch_ao_mo_x2(d, walkers, W, ldw, v, nch, st)
-                                 : launch_ao_mo_simt(d, wf->precision, walkers, W, ldw, v, nch, st),
+                                 : launch_ao_mo_simt(d, wf->precision, walkers, W, ldw, v, nch,
+                                                     averaged || d.n_det == 1, st),
                     "ao_mo");
   if (s) return s;
   mark(wf, 3, st);
@@ -1427,7 +1428,7 @@ qmc_status qmc_energy_grad(qmc_wf* wf, const double* walkers, int64_t n_walkers,
   s = small ? launch_status(launch_small_grad(wf->dev, walkers, n_walkers, ldw, wf->dev.ao_prim, n_prim, e_loc,
                                               partial, st),
                             "energies and gradient sums")
-            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
+            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st, nullptr, nullptr, true);
   if (s) return s;
   s = launch_status(launch_mean_var(e_loc, n_walkers, stats, st), "mean/variance");
   if (s) return s;
@@ -1484,7 +1485,7 @@ qmc_status qmc_energy_grad_sums(qmc_wf* wf, const double* walkers, int64_t n_wal
   s = small ? launch_status(launch_small_grad(wf->dev, walkers, n_walkers, ldw, wf->dev.ao_prim, n_prim, e_loc,
                                               partial, st),
                             "energies and gradient sums")
-            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st);
+            : eval_path(wf, walkers, n_walkers, ldw, ws, err_flag, true, e_loc, nullptr, st, nullptr, nullptr, true);
   if (s) return s;
   s = launch_status(launch_energy_sums(e_loc, n_walkers, sums, st), "energy sums");
   if (s) return s;

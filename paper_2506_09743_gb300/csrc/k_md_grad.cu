@@ -29,10 +29,10 @@
 // tables, CI sum, Gamma, the CI-weight and Jastrow terms) writes Gamma to
 // scratch; k_md_rows (one thread per electron row) evaluates the AOs and
 // adds the coefficient, exponent and backflow terms.  Per-walker values are
-// weighted (estimator 2 (E_L - E_v) / M, one, or E_L) and summed per warp by
-// shuffles in a fixed order (a butterfly reduce-scatter for the outputs of
-// two AOs at a time), per block over the warps in order, and over the blocks
-// by k_row_sums: the result is bitwise reproducible.
+// weighted (estimator 2 (E_L - E_v) / M, one, or E_L) and summed per warp in a
+// fixed order, per block over the warps in order, and over the blocks by
+// k_row_sums: the result is bitwise reproducible.
+#include "fp64_math.cuh"
 #include "general_eval.cuh"
 
 namespace qmc {
@@ -57,12 +57,12 @@ __device__ __forceinline__ double walker_weight(int weight, const double* e_loc,
   return 2.0 * (e_loc[w] - stats[0]) / (double)W;
 }
 
-// per-warp accumulators [kMdWarps][n_param] -> partial[k][col] in a fixed order
+// per-warp accumulators [warps][n_param] -> partial[k][col] in a fixed order
 __device__ void flush_acc(const double* acc, int n_param, double* partial, int64_t ld_partial, int col) {
   __syncthreads();
   for (int k = threadIdx.x; k < n_param; k += blockDim.x) {
     double s = 0.0;
-    for (int q = 0; q < kMdWarps; ++q) s += acc[(size_t)q * n_param + k];
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += acc[(size_t)q * n_param + k];
     partial[(size_t)k * ld_partial + col] = s;
   }
 }
@@ -252,149 +252,206 @@ __global__ void __launch_bounds__(kMdThreads) k_md_gamma(WfDev wf, const double*
   flush_acc(acc, n_param, partial, ld_partial, blockIdx.x);
 }
 
-// Sum over the warp's lanes of 32 values per lane: afterwards lane L holds the
-// sum of every lane's v[L].  Butterfly reduce-scatter in five exchange
-// stages (31 adds per lane for 32 outputs, instead of five per output for a
-// per-output tree); the order of the additions is fixed.
-__device__ __forceinline__ double reduce_scatter32(double (&v)[32], int lane) {
-#pragma unroll
-  for (int s = 16; s >= 1; s >>= 1) {
-    const bool upper = (lane & s) != 0;
-#pragma unroll
-    for (int k = 0; k < s; ++k) {
-      const double send = upper ? v[k] : v[k + s];
-      const double keep = upper ? v[k + s] : v[k];
-      v[k] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-    }
-  }
-  return v[0];
-}
+// Row kernel.  It is bound by the FP64 pipe, so the split minimises FP64
+// instructions: 65,536 CO walkers took 16.6 ms when every coefficient and
+// exponent value was formed per row and summed over the warp by shuffles (about
+// 95 instructions per AO and row).  A warp takes 32 rows of one electron, and
+//   1. each lane evaluates its row's AOs, a chunk of up to kChunkAo at a time:
+//      values phi_b, the weighted exponent factors q_b = w u_b P_b and the
+//      shells' radial derivatives go to shared memory;
+//   2. the chunk's outputs are then formed as sums over the 32 rows,
+//        C: sum_r phi_b[r] (w Gamma_m)[r],   alpha: sum_r q_b[r] (d f/d alpha_p)[r],
+//      one output per lane and round, one FMA per row (the reduction over the
+//      rows is the FMA chain itself), added to the warp's sums in shared memory.
+// Rows, chunks, warps and blocks are taken in a fixed order.
+constexpr int kChunkAo = 16;
+constexpr int kChunkRad = 24;   // radial derivatives (shells x primitives) of a chunk
+constexpr int kRowPad = 33;
 
-__global__ void __launch_bounds__(kMdThreads) k_md_rows(WfDev wf, const double* __restrict__ walkers, int64_t W,
-                                                         int64_t ldw, const double* __restrict__ gam, int64_t ldm,
+// doubles of a warp's chunk buffers: phi, q, w Gamma, radial derivatives
+constexpr int kRowsBuf = (2 * kChunkAo + kMdNM + kChunkRad) * kRowPad;
+
+__global__ void __launch_bounds__(kMdThreads) k_md_rows(const __grid_constant__ WfDev wf,
+                                                         const double* __restrict__ walkers, int64_t W, int64_t ldw,
+                                                         const double* __restrict__ gam, int64_t ldm,
                                                          const double* __restrict__ e_loc,
                                                          const double* __restrict__ stats, int weight,
                                                          const double* __restrict__ ang,
                                                          const int* __restrict__ prim_start, int n_param,
                                                          double* __restrict__ partial, int64_t ld_partial, int col0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  GenShared g;
-  stage_tables(wf, g, smem_raw);
-  const size_t tab_bytes = (sizeof(ShellDev) * wf.n_shell + sizeof(int) * wf.n_ao + 15) & ~size_t(15);
-  double* acc = reinterpret_cast<double*>(smem_raw + tab_bytes);  // [kMdWarps][n_param]
-  for (int k = threadIdx.x; k < kMdWarps * n_param; k += blockDim.x) acc[k] = 0.0;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, n_warp = blockDim.x >> 5;
+  const int N = wf.n_elec, nmo = wf.n_mo, n_ao = wf.n_ao;
+  const int n_prim = prim_start[n_ao];
+  const int off_c = n_prim, off_w = off_c + n_ao * nmo + wf.n_det + 1;
+  double* acc = reinterpret_cast<double*>(smem_raw);                      // [n_warp][n_param]
+  double* buf = acc + (size_t)n_warp * n_param + (size_t)warp * kRowsBuf;
+  // exponent parameter -> AO within its chunk << 8 | radial derivative within the chunk
+  unsigned short* slot = reinterpret_cast<unsigned short*>(acc + (size_t)n_warp * (n_param + kRowsBuf));
+  double* phi_s = buf;                           // [kChunkAo][33]
+  double* q_s = phi_s + kChunkAo * kRowPad;      // [kChunkAo][33]
+  double* wg_s = q_s + kChunkAo * kRowPad;       // [kMdNM][33]
+  double* rd_s = wg_s + kMdNM * kRowPad;         // [kChunkRad][33]
+  for (int k = threadIdx.x; k < n_warp * n_param; k += blockDim.x) acc[k] = 0.0;
+  // chunk of shell s: consecutive shells while their AOs and radial
+  // derivatives fit (the same rule in the loop below)
+  auto fits = [&](int ao, int rad, const ShellDev& sh) {
+    return ao == 0 || (ao + sh.n_ao <= kChunkAo && rad + sh.n_prim <= kChunkRad);
+  };
+  if (threadIdx.x == 0) {
+    int ao = 0, rad = 0;
+    for (int s = 0; s < wf.n_shell; ++s) {
+      const ShellDev& sh = wf.shells[s];
+      if (!fits(ao, rad, sh)) ao = rad = 0;
+      for (int k = 0; k < sh.n_ao; ++k)
+        for (int p = 0; p < sh.n_prim; ++p)
+          slot[prim_start[sh.ao_first + k] + p] = (unsigned short)(((ao + k) << 8) | (rad + p));
+      ao += sh.n_ao;
+      rad += sh.n_prim;
+    }
+  }
   __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int N = wf.n_elec, nmo = wf.n_mo;
-  const int n_prim = prim_start[wf.n_ao];
-  const int off_c = n_prim, off_w = off_c + wf.n_ao * nmo + wf.n_det + 1;
   double* my = acc + (size_t)warp * n_param;
-  const int64_t rows = (int64_t)N * W;
-  const int64_t n_iter = (rows + (int64_t)gridDim.x * kMdThreads - 1) / ((int64_t)gridDim.x * kMdThreads);
-  for (int64_t it = 0; it < n_iter; ++it) {
-    const int64_t q = (it * gridDim.x + blockIdx.x) * kMdThreads + threadIdx.x;
-    const bool live = q < rows;
-    const int i = live ? (int)(q / W) : 0;
-    const int64_t w = live ? q % W : 0;
+  const int64_t n_tile = (W + 31) / 32;  // tiles of 32 walkers, per electron
+  const int64_t n_work = n_tile * N;
+  for (int64_t t = (int64_t)blockIdx.x * n_warp + warp; t < n_work; t += (int64_t)gridDim.x * n_warp) {
+    const int i = (int)(t / n_tile);
+    const int64_t w0 = (t - (int64_t)i * n_tile) * 32 + lane;
+    const bool live = w0 < W;
+    const int64_t w = live ? w0 : W - 1;
     const double wt = live ? walker_weight(weight, e_loc, stats, w, W) : 0.0;
     double r[3], drt[3] = {0.0, 0.0, 0.0};
     for (int c = 0; c < 3; ++c) r[c] = walkers[(int64_t)(3 * i + c) * ldw + w];
     for (int j = 0; j < N; ++j) {
       if (j == i) continue;
-      double v[3], d2 = 0.0;
-      for (int c = 0; c < 3; ++c) {
-        v[c] = r[c] - walkers[(int64_t)(3 * j + c) * ldw + w];
-        d2 += v[c] * v[c];
-      }
-      const double inv = 1.0 / sqrt(d2);
-      for (int c = 0; c < 3; ++c) drt[c] += inv * v[c];
+      double v[3];
+      for (int c = 0; c < 3; ++c) v[c] = r[c] - walkers[(int64_t)(3 * j + c) * ldw + w];
+      const double inv = rsqrt3(fma(v[2], v[2], fma(v[1], v[1], v[0] * v[0])));
+      for (int c = 0; c < 3; ++c) drt[c] = fma(inv, v[c], drt[c]);
     }
     double G[kMdNM];
-    for (int m = 0; m < kMdNM; ++m) G[m] = (live && m < nmo) ? gam[((size_t)i * nmo + m) * ldm + w] : 0.0;
+#pragma unroll
+    for (int m = 0; m < kMdNM; ++m) {
+      G[m] = m < nmo ? gam[((size_t)i * nmo + m) * ldm + w] : 0.0;
+      wg_s[m * kRowPad + lane] = wt * G[m];
+    }
     double gw = 0.0;
-    for (int s = 0; s < wf.n_shell; ++s) {
-      const ShellDev& sh = g.sh[s];
-      const double dx = r[0] - wf.atom_xyz[sh.atom][0], dy = r[1] - wf.atom_xyz[sh.atom][1],
-                   dz = r[2] - wf.atom_xyz[sh.atom][2];
-      const double r2 = dx * dx + dy * dy + dz * dz, rho = sqrt(r2);
-      // radial factor, f'/rho, and per primitive the exponent derivative of
-      // its normalised term: d(N_p e^(-alpha r^2)) / d alpha = term ((3/4 + l/2)/alpha - r^2)
-      double f = 0.0, g1 = 0.0, dexp[QMC_MAX_PRIM];
-      if (sh.kind == 0) {
-        double rk = 1.0;
-        for (int k = 0; k < sh.kn; ++k) rk *= rho;
-        f = sh.coef[0] * rk * exp(-sh.expo[0] * rho);
-        g1 = (sh.kn / rho - sh.expo[0]) * f / rho;
-        const int nq = sh.kn + sh.l + 1;
-        dexp[0] = f * ((nq + 0.5) / sh.expo[0] - rho);
-      } else {
-        for (int p = 0; p < sh.n_prim; ++p) {
-          const double al = sh.expo[p];
-          const double term = sh.coef[p] * exp(-al * r2);
-          f += term;
-          g1 -= 2.0 * al * term;
-          dexp[p] = term * ((0.75 + 0.5 * sh.l) / al - r2);
+    int cur_atom = -1;
+    double dv[3] = {0.0, 0.0, 0.0}, r2 = 0.0, rho = 0.0, irho = 0.0, D = 0.0;
+    for (int s0 = 0; s0 < wf.n_shell;) {
+      int ao = 0, rad = 0, s = s0;
+      const int b0 = wf.shells[s0].ao_first;
+      for (; s < wf.n_shell; ++s) {
+        const ShellDev& sh = wf.shells[s];
+        if (!fits(ao, rad, sh)) break;
+        if (sh.atom != cur_atom) {
+          cur_atom = sh.atom;
+          for (int c = 0; c < 3; ++c) dv[c] = r[c] - wf.atom_xyz[cur_atom][c];
+          r2 = fma(dv[2], dv[2], fma(dv[1], dv[1], dv[0] * dv[0]));
+          D = fma(dv[2], drt[2], fma(dv[1], drt[1], dv[0] * drt[0]));
+          if (wf.any_sto) {
+            irho = rsqrt3(r2);
+            rho = sqrt_from(r2, irho);
+          }
         }
-      }
-      const double dv[3] = {dx, dy, dz};
-      // AOs two at a time: MO-coefficient terms of AO k in slots [16 (k & 1), +16)
-      for (int k0 = 0; k0 < sh.n_ao; k0 += 2) {
-        double vc[32];
-        double ub[2] = {0.0, 0.0}, Pm[2] = {0.0, 0.0};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = k0 + h;
-          const bool has = k < sh.n_ao;
-          const int b = has ? sh.ao_first + k : sh.ao_first;
-          const int pw = g.pw[b];
+        // radial factor, f'/rho, and per primitive the exponent derivative of
+        // its normalised term: d(N_p e^(-alpha r^2))/d alpha = term ((3/4 + l/2)/alpha - r^2)
+        const double* nak = wf.nak + (size_t)s * QMC_MAX_PRIM;
+        double f = 0.0, g1 = 0.0;
+        if (sh.kind == 0) {
+          f = sh.coef[0] * exp_scaled(nak[0], rho, wf.exp2_tab);
+          for (int k = 0; k < sh.kn; ++k) f *= rho;
+          g1 = fma((double)sh.kn, irho, -sh.expo[0]) * f * irho;
+          rd_s[rad * kRowPad + lane] = f * (((double)(sh.kn + sh.l + 1) + 0.5) * recip3(sh.expo[0]) - rho);
+        } else {
+          for (int p = 0; p < sh.n_prim; ++p) {
+            const double al = sh.expo[p];
+            const double term = sh.coef[p] * exp_scaled(nak[p], r2, wf.exp2_tab);
+            f += term;
+            g1 = fma(nak[p], term, g1);  // -2048 alpha / ln 2, scaled below
+            rd_s[(rad + p) * kRowPad + lane] = term * fma(0.75 + 0.5 * sh.l, recip3(al), -r2);
+          }
+          g1 *= 2.0 * (0.69314718055994530942 / 2048.0);
+        }
+        const double h = g1 * D;
+        for (int k = 0; k < sh.n_ao; ++k) {
+          const int b = sh.ao_first + k;
+          const int pw = wf.ao_pow[b];
           const int pa[3] = {pw & 15, (pw >> 4) & 15, (pw >> 8) & 15};
-          Pm[h] = has ? mono(dx, dy, dz, pa[0], pa[1], pa[2]) : 0.0;
-          const double sb = wt * ang[b] * Pm[h] * f;
-          const double* Cb = g.C + (size_t)b * nmo;  // angular factor folded in
-          double u = 0.0;
-#pragma unroll
-          for (int m = 0; m < kMdNM; ++m) {
-            vc[16 * h + m] = sb * G[m];
-            if (m < nmo) u += Cb[m] * G[m];
+          // P and grad(P f) . drt = f grad P . drt + P g1 (v . drt)
+          double P, gd;
+          if (sh.l == 0) {
+            P = 1.0;
+            gd = h;
+          } else if (sh.l == 1) {
+            const bool px = pa[0] != 0, py = pa[1] != 0;
+            P = px ? dv[0] : py ? dv[1] : dv[2];
+            gd = fma(P, h, f * (px ? drt[0] : py ? drt[1] : drt[2]));
+          } else if (sh.l == 2) {
+            const int c = pa[0] ? 0 : pa[1] ? 1 : 2;                  // first factor
+            const int e = pa[c] == 2 ? c : (pa[2] ? 2 : 1);           // second
+            const double vc = c == 0 ? dv[0] : c == 1 ? dv[1] : dv[2], ve = e == 0 ? dv[0] : e == 1 ? dv[1] : dv[2];
+            const double tc = c == 0 ? drt[0] : c == 1 ? drt[1] : drt[2],
+                         te = e == 0 ? drt[0] : e == 1 ? drt[1] : drt[2];
+            P = vc * ve;
+            gd = fma(P, h, f * fma(vc, te, ve * tc));
+          } else {
+            P = mono(dv[0], dv[1], dv[2], pa[0], pa[1], pa[2]);
+            double dP = 0.0;
+            for (int c = 0; c < 3; ++c)
+              if (pa[c] > 0)
+                dP += pa[c] * mono(dv[0], dv[1], dv[2], pa[0] - (c == 0), pa[1] - (c == 1), pa[2] - (c == 2)) * drt[c];
+            gd = fma(P, h, f * dP);
           }
-          ub[h] = has ? u : 0.0;
-          // grad (P f) . sum_j (r_a - r_j) / r_aj
-          if (has) {
-            double gd = 0.0;
-            for (int d = 0; d < 3; ++d) {
-              double dP = 0.0;
-              if (pa[d] > 0) {
-                const int e[3] = {pa[0] - (d == 0), pa[1] - (d == 1), pa[2] - (d == 2)};
-                dP = pa[d] * mono(dx, dy, dz, e[0], e[1], e[2]);
-              }
-              gd += (f * dP + Pm[h] * g1 * dv[d]) * drt[d];
-            }
-            gw += u * gd;
+          const double* Cb = wf.mo64 + (size_t)b * nmo;  // angular factor folded in
+          double u0 = 0.0, u1 = 0.0;
+#pragma unroll
+          for (int m = 0; m < kMdNM; m += 2) {
+            if (m < nmo) u0 = fma(__ldg(Cb + m), G[m], u0);
+            if (m + 1 < nmo) u1 = fma(__ldg(Cb + m + 1), G[m + 1], u1);
           }
+          const double u = u0 + u1;
+          phi_s[(ao + k) * kRowPad + lane] = P * f;
+          q_s[(ao + k) * kRowPad + lane] = wt * u * P;
+          gw = fma(u, gd, gw);
         }
-        const double oc = reduce_scatter32(vc, lane);
-        {
-          const int k = k0 + (lane >> 4), m = lane & 15;
-          if (k < sh.n_ao && m < nmo) my[off_c + (sh.ao_first + k) * nmo + m] += oc;
-        }
-        // exponent terms of the same two AOs: slots [8 h + p]
-        double ve[32];
-#pragma unroll
-        for (int t = 0; t < 32; ++t) ve[t] = 0.0;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const double qb = wt * ub[h] * Pm[h];
-          for (int p = 0; p < sh.n_prim && p < QMC_MAX_PRIM; ++p) ve[8 * h + p] = qb * dexp[p];
-        }
-        const double oe = reduce_scatter32(ve, lane);
-        {
-          const int h = lane >> 3, p = lane & 7, k = k0 + h;
-          if (h < 2 && k < sh.n_ao && p < (sh.kind == 0 ? 1 : sh.n_prim)) my[prim_start[sh.ao_first + k] + p] += oe;
-        }
+        ao += sh.n_ao;
+        rad += sh.n_prim;
       }
+      __syncwarp();
+      // coefficients of the chunk's AOs (angular factor applied here)
+      const int n_c = ao * nmo;
+      for (int o = lane; o < n_c; o += 32) {
+        const int b = o / nmo, m = o - b * nmo;
+        const double* x = phi_s + b * kRowPad;
+        const double* y = wg_s + m * kRowPad;
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < 32; q += 2) {
+          a0 = fma(x[q], y[q], a0);
+          a1 = fma(x[q + 1], y[q + 1], a1);
+        }
+        my[off_c + b0 * nmo + o] = fma(ang[b0 + b], a0 + a1, my[off_c + b0 * nmo + o]);
+      }
+      // exponents of the chunk's primitives
+      const int p1 = prim_start[b0 + ao];
+      for (int o = prim_start[b0] + lane; o < p1; o += 32) {
+        const double* x = q_s + (slot[o] >> 8) * kRowPad;
+        const double* y = rd_s + (slot[o] & 0xff) * kRowPad;
+        double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+        for (int q = 0; q < 32; q += 2) {
+          a0 = fma(x[q], y[q], a0);
+          a1 = fma(x[q + 1], y[q + 1], a1);
+        }
+        my[o] += a0 + a1;
+      }
+      __syncwarp();
+      s0 = s;
     }
     const double v = warp_sum(wt * gw);
     if (lane == 0) my[off_w] += v;
+    __syncwarp();
   }
   flush_acc(acc, n_param, partial, ld_partial, col0 + blockIdx.x);
 }
@@ -404,6 +461,11 @@ bool md_grad_supported(const WfDev& wf) {
   const int ns = wf.n_up > wf.n_down ? wf.n_up : wf.n_down;
   if (ns > kMdNS || wf.n_mo > kMdNM || wf.n_exc[0] > 128 || wf.n_exc[1] > 128) return false;
   return true;
+}
+
+// shared memory of k_md_rows with n warps per block
+static size_t md_rows_smem_bytes(int n_prim, int n_param, int n) {
+  return sizeof(double) * n * ((size_t)n_param + kRowsBuf) + ((sizeof(unsigned short) * (size_t)n_prim + 15) & ~size_t(15));
 }
 
 size_t md_grad_smem_bytes(const WfDev& wf, int n_param) {
@@ -436,10 +498,14 @@ cudaError_t launch_md_grad(const WfDev& wf, const double* walkers, int64_t W, in
                                              n_param, off_d, gam, partial, ldp);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  const size_t smem_b = md_grad_smem_bytes(wf, n_param);
+  // warps per block: four (two blocks of them per SM for CO's 1,008
+  // parameters), fewer where a warp's parameter sums are too many
+  int warps = kMdWarps;
+  while (warps > 1 && md_rows_smem_bytes(n_prim, n_param, warps) > 227 * 1024) warps /= 2;
+  const size_t smem_b = md_rows_smem_bytes(n_prim, n_param, warps);
   e = cudaFuncSetAttribute(k_md_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_b);
   if (e != cudaSuccess) return e;
-  k_md_rows<<<nb, kMdThreads, smem_b, st>>>(wf, walkers, W, ldw, gam, ws.ldm, e_loc, stats, weight, wf.ao_ang,
+  k_md_rows<<<nb, 32 * warps, smem_b, st>>>(wf, walkers, W, ldw, gam, ws.ldm, e_loc, stats, weight, wf.ao_ang,
                                             wf.ao_prim, n_param, partial, ldp, nb);
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -336,7 +336,7 @@ size_t een_shared_bytes(const WfDev& wf, bool fp64);
 cudaError_t launch_jastrow(const WfDev& wf, int prec, const double* walkers, int64_t W, int64_t ldw, double* copy,
                            const Workspace& ws, bool derivs, cudaStream_t st);
 cudaError_t launch_ao_mo_simt(const WfDev& wf, int prec, const double* walkers, int64_t W, int64_t ldw,
-                              const Workspace& ws, int nch, cudaStream_t st);
+                              const Workspace& ws, int nch, bool fast, cudaStream_t st);
 // pairs of FP32 (QMC_FP32X2 form): SIMT contraction, and the digit-sliced
 // tensor-core contraction where oz_supported
 size_t oz_smem_bytes(const WfDev& wf, int nch, int groups);

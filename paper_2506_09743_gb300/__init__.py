@@ -34,14 +34,16 @@ def _stream_handle(stream):
     if stream is None:
         import torch
 
-        return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+        # the raw handle of the current device's current stream, without the
+        # stream object that torch.cuda.current_stream() builds on each call
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return ctypes.c_void_p(stream)
     return ctypes.c_void_p(stream.cuda_stream)
 
 
 def _dptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 class Wavefunction:

@@ -43,6 +43,52 @@ namespace {
 
 constexpr int kWalkersPerBlock = 32;  // 64 threads: (walker, spin) pairs
 
+// cof[r][m] = cofactor of a[r][m]
+template <int NS>
+__device__ __forceinline__ void cofactor_matrix(const double (&a)[NS][NS], double (&cof)[NS][NS]) {
+  if constexpr (NS == 1) {
+    cof[0][0] = 1.0;
+  } else if constexpr (NS == 2) {
+    cof[0][0] = a[1][1];
+    cof[0][1] = -a[1][0];
+    cof[1][0] = -a[0][1];
+    cof[1][1] = a[0][0];
+  } else if constexpr (NS == 3) {
+#pragma unroll
+    for (int r = 0; r < 3; ++r)
+#pragma unroll
+      for (int m = 0; m < 3; ++m) {
+        const int r1 = (r + 1) % 3, r2 = (r + 2) % 3, m1 = (m + 1) % 3, m2 = (m + 2) % 3;
+        cof[r][m] = fma(a[r1][m1], a[r2][m2], -(a[r1][m2] * a[r2][m1]));
+      }
+  } else {
+    // 2x2 minors of the upper and lower row pairs, then Laplace expansions
+    double u[4][4], l[4][4];
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int d = c + 1; d < 4; ++d) {
+        u[c][d] = fma(a[0][c], a[1][d], -(a[0][d] * a[1][c]));
+        l[c][d] = fma(a[2][c], a[3][d], -(a[2][d] * a[3][c]));
+      }
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        int c[3], k = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q != m) c[k++] = q;
+        // the partner row in r's own pair, the other pair's minors
+        const int o = r ^ 1;
+        double v;
+        if (r < 2) v = fma(a[o][c[0]], l[c[1]][c[2]], fma(-a[o][c[1]], l[c[0]][c[2]], a[o][c[2]] * l[c[0]][c[1]]));
+        else v = fma(a[o][c[0]], u[c[1]][c[2]], fma(-a[o][c[1]], u[c[0]][c[2]], a[o][c[2]] * u[c[0]][c[1]]));
+        cof[r][m] = ((r + m) & 1) ? -v : v;
+      }
+  }
+}
+
 }  // namespace
 
 template <int NS, bool KIN>
@@ -252,7 +298,60 @@ __global__ void __launch_bounds__(2 * kWalkersPerBlock)
   }
 }
 
+// One determinant and at most four electrons per spin (H2, LiH): no tables, so
+// one thread takes both spins of a walker, with the inverse from cofactors.
+// The kernel is bound by the FP64 pipe: per warp of 32 walkers about 60
+// instructions at two electrons per spin (half of them the logarithm), where
+// k_det's thread pair spends about 115 per 16 walkers.
+template <int NS, bool KIN>
+__global__ void __launch_bounds__(128) k_det_one(const __grid_constant__ WfDev wf, int64_t W,
+                                                 const double* __restrict__ mo, int nmp, int64_t ldm,
+                                                 const double* __restrict__ jscal, double* __restrict__ e_loc,
+                                                 double* __restrict__ log_psi) {
+  constexpr int NCH = KIN ? 2 : 1;
+  const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (w >= W) return;
+  double det = wf.det_w[0], tr = 0.0;
+#pragma unroll
+  for (int s = 0; s < 2; ++s) {
+    const int n = s == 0 ? wf.n_up : wf.n_down, i0 = s == 0 ? 0 : wf.n_up;
+    if (n == 0) continue;
+    auto ld = [&](int c, int r, int m) { return mo[((int64_t)((i0 + r) * NCH + c) * nmp + m) * ldm + w]; };
+    double a[NS][NS];
+#pragma unroll
+    for (int r = 0; r < NS; ++r)
+#pragma unroll
+      for (int m = 0; m < NS; ++m) a[r][m] = (r < n && m < n) ? ld(0, r, m) : (r == m ? 1.0 : 0.0);
+    double cof[NS][NS];
+    cofactor_matrix<NS>(a, cof);
+    double d = a[0][0] * cof[0][0];
+#pragma unroll
+    for (int m = 1; m < NS; ++m) d = fma(a[0][m], cof[0][m], d);
+    if (KIN) {
+      double t = 0.0;
+#pragma unroll
+      for (int r = 0; r < NS; ++r)
+#pragma unroll
+        for (int m = 0; m < NS; ++m)
+          if (r < n && m < n) t = fma(cof[r][m], ld(1, r, m), t);
+      tr = fma(t, recip(d), tr);
+    }
+    det *= d;
+  }
+  if (log_psi) log_psi[w] = jscal[w] + log(fabs(det));
+  if (KIN) e_loc[w] = -0.5 * (jscal[ldm + w] + tr) + jscal[2 * ldm + w];
+}
+
 namespace {
+
+template <int NS>
+cudaError_t launch_one(const WfDev& wf, int64_t W, const Workspace& ws, bool kin, double* e_loc, double* log_psi,
+                       cudaStream_t st) {
+  const unsigned grid = (unsigned)((W + 127) / 128);
+  if (kin) k_det_one<NS, true><<<grid, 128, 0, st>>>(wf, W, ws.mo, ws.nmp, ws.ldm, ws.jscal, e_loc, log_psi);
+  else k_det_one<NS, false><<<grid, 128, 0, st>>>(wf, W, ws.mo, ws.nmp, ws.ldm, ws.jscal, e_loc, log_psi);
+  return cudaGetLastError();
+}
 
 // doubles of tables per walker in shared memory, made odd so that the 32
 // walkers of a block start on different banks (the threads of a warp read
@@ -286,6 +385,14 @@ cudaError_t launch_det(const WfDev& wf, int prec, int64_t W, const Workspace& ws
   (void)prec;  // the MO channels are FP64 in every form
   if (W == 0) return cudaSuccess;
   const int ns = wf.n_up > wf.n_down ? wf.n_up : wf.n_down;
+  if (wf.n_det == 1 && wf.n_col == ns) {  // the ground determinant alone
+    switch (ns) {
+      case 1: return launch_one<1>(wf, W, ws, kinetic, e_loc, log_psi, st);
+      case 2: return launch_one<2>(wf, W, ws, kinetic, e_loc, log_psi, st);
+      case 3: return launch_one<3>(wf, W, ws, kinetic, e_loc, log_psi, st);
+      case 4: return launch_one<4>(wf, W, ws, kinetic, e_loc, log_psi, st);
+    }
+  }
   switch (ns) {
     case 1: return launch_ns<1>(wf, W, ws, kinetic, e_loc, log_psi, st);
     case 2: return launch_ns<2>(wf, W, ws, kinetic, e_loc, log_psi, st);

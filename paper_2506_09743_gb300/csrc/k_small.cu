@@ -13,19 +13,47 @@ cudaError_t box_muller_tables(BmTables* t);
 
 namespace {
 
-// Warps are the unit of work: one-warp blocks spread a small batch over all SM
-// partitions evenly.
+// Warps are the unit of work.  FP64: one-warp blocks spread a small batch over
+// all SM partitions evenly, and the tables are read through L1 (their latency
+// hides behind the FP64 pipe).  Pairs of FP32: the orbitals are bound by latency
+// and issue, so four warps share tables staged in shared memory.
 constexpr int kBlock = 32;
+constexpr int kBlockPairs = 128;
+
+// the orbital tables: in global memory, or (STAGE) copied to the block's
+// dynamic shared memory
+size_t table_bytes(const WfDev& wf) {
+  return sizeof(ShellDev) * (size_t)wf.n_shell + sizeof(float2) * (size_t)wf.n_ao * wf.n_mo + sizeof(float) * 128;
+}
+
+template <bool STAGE>
+__device__ __forceinline__ Tables tables(const WfDev& wf) {
+  if constexpr (!STAGE) {
+    return Tables{wf.shells, wf.mo_x2, wf.exp_tab};
+  } else {
+    extern __shared__ __align__(16) unsigned char tab_raw[];
+    ShellDev* sh = reinterpret_cast<ShellDev*>(tab_raw);
+    float2* C = reinterpret_cast<float2*>(sh + wf.n_shell);
+    float* ex = reinterpret_cast<float*>(C + (size_t)wf.n_ao * wf.n_mo);
+    for (int k = threadIdx.x; k < wf.n_shell * (int)(sizeof(ShellDev) / 4); k += blockDim.x)
+      reinterpret_cast<int*>(sh)[k] = reinterpret_cast<const int*>(wf.shells)[k];
+    for (int k = threadIdx.x; k < wf.n_ao * wf.n_mo; k += blockDim.x) C[k] = wf.mo_x2[k];
+    for (int k = threadIdx.x; k < 128; k += blockDim.x) ex[k] = wf.exp_tab[k];
+    __syncthreads();
+    return Tables{sh, C, ex};
+  }
+}
 
 }  // namespace
 
 template <int NE, int NO, bool BF, bool PAIRS>
-__global__ void __launch_bounds__(kBlock, PAIRS ? 12 : 1) k_small_energy(const __grid_constant__ WfDev wf,
+__global__ void __launch_bounds__(PAIRS ? kBlockPairs : kBlock, PAIRS ? 3 : 1) k_small_energy(const __grid_constant__ WfDev wf,
                                                          const double* __restrict__ walkers, int64_t W, int64_t ldw,
                                                          double* __restrict__ e_loc, double* __restrict__ log_psi) {
   constexpr int MODE = BF ? 2 : 1;
   using U = typename std::conditional<PAIRS, f32x2, double>::type;
-  const Group g = make_group(wf.n_elec, blockIdx.x, W);
+  const Tables tb = tables<PAIRS>(wf);
+  const Group g = make_group(wf.n_elec, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), W);
   const int N = g.N, nu = wf.n_up;
   const int s = g.e >= nu ? 1 : 0, n = s ? wf.n_down : nu, i0 = s ? nu : 0, a = g.e - i0;
   double r[3];
@@ -40,7 +68,7 @@ __global__ void __launch_bounds__(kBlock, PAIRS ? 12 : 1) k_small_energy(const _
 
   // ---- orbitals, this electron's column of the inverse
   Mo<NO, MODE> mo;
-  orbitals<U, NO, MODE>(wf, rt, mo);
+  orbitals<U, NO, MODE>(wf, tb, rt, mo);
   double ai[NO];
   const double det = cofactors<NO>(g, mo.phi, a, n, i0, ai);
   const double idet = recip3(det);
@@ -158,13 +186,14 @@ __global__ void __launch_bounds__(kBlock, PAIRS ? 12 : 1) k_small_energy(const _
 // coordinates by shuffles.  The acceptance test u < |Psi'/Psi|^2 is made on the
 // ratio of the determinants and exp(2 (J' - J)), so a step takes no logarithm.
 template <int NE, int NO, bool BF, bool PAIRS>
-__global__ void __launch_bounds__(kBlock) k_small_chain(const __grid_constant__ WfDev wf, double* __restrict__ walkers,
+__global__ void __launch_bounds__(PAIRS ? kBlockPairs : kBlock) k_small_chain(const __grid_constant__ WfDev wf, double* __restrict__ walkers,
                                                         int64_t W, int64_t ldw, int n_steps, double step,
                                                         uint64_t seed, uint64_t first_walker, uint64_t step0,
                                                         BmTables bm, double* __restrict__ log_psi,
                                                         int64_t* __restrict__ n_accept) {
   using U = typename std::conditional<PAIRS, f32x2, double>::type;
-  const Group g = make_group(wf.n_elec, blockIdx.x, W);
+  const Tables tb = tables<PAIRS>(wf);
+  const Group g = make_group(wf.n_elec, blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), W);
   const int N = g.N, nu = wf.n_up;
   const int s = g.e >= nu ? 1 : 0, n = s ? wf.n_down : nu, i0 = s ? nu : 0, a = g.e - i0;
   const int n3 = 3 * N, n_pairs = (n3 + 1) / 2;
@@ -241,7 +270,7 @@ __global__ void __launch_bounds__(kBlock) k_small_chain(const __grid_constant__ 
 #pragma unroll
     for (int d = 0; d < 3; ++d) rt[d] = BF ? fma(wf.bf_w, drt[d], q[d]) : q[d];
     Mo<NO, 0> mo;
-    orbitals<U, NO, 0>(wf, rt, mo);
+    orbitals<U, NO, 0>(wf, tb, rt, mo);
     double cof[NO];
     const double dn = cofactors<NO>(g, mo.phi, a, n, i0, cof);
     Jn = shfl(group_sum<NE>(g, Jn), g.base);
@@ -288,7 +317,11 @@ cudaError_t launch_small_energy(const WfDev& wf, const double* walkers, int64_t 
   if (wf.bf_w == 0.0) {
     QMC_SMALL_DISPATCH((k_small_energy<NE, NO, false, false><<<grid, kBlock, 0, st>>>(wf, walkers, W, ldw, e_loc, log_psi)));
   } else if (wf.gen_x2) {
-    QMC_SMALL_DISPATCH((k_small_energy<NE, NO, true, true><<<grid, kBlock, 0, st>>>(wf, walkers, W, ldw, e_loc, log_psi)));
+    const size_t tb = table_bytes(wf);
+    QMC_SMALL_DISPATCH((cudaFuncSetAttribute(k_small_energy<NE, NO, true, true>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tb),
+                        k_small_energy<NE, NO, true, true><<<(grid + 3) / 4, kBlockPairs, tb, st>>>(
+                            wf, walkers, W, ldw, e_loc, log_psi)));
   } else {
     QMC_SMALL_DISPATCH((k_small_energy<NE, NO, true, false><<<grid, kBlock, 0, st>>>(wf, walkers, W, ldw, e_loc, log_psi)));
   }
@@ -316,7 +349,10 @@ cudaError_t launch_small_chain(const WfDev& wf, double* walkers, int64_t W, int6
       QMC_SMALL_DISPATCH((k_small_chain<NE, NO, false, false><<<grid, kBlock, 0, st>>>(
           wf, walkers, W, ldw, nt, step, seed, first_walker, off, bm, lp, n_accept)));
     } else if (wf.gen_x2) {
-      QMC_SMALL_DISPATCH((k_small_chain<NE, NO, true, true><<<grid, kBlock, 0, st>>>(
+      const size_t tb = table_bytes(wf);
+      QMC_SMALL_DISPATCH((cudaFuncSetAttribute(k_small_chain<NE, NO, true, true>,
+                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tb),
+                          k_small_chain<NE, NO, true, true><<<(grid + 3) / 4, kBlockPairs, tb, st>>>(
           wf, walkers, W, ldw, nt, step, seed, first_walker, off, bm, lp, n_accept)));
     } else {
       QMC_SMALL_DISPATCH((k_small_chain<NE, NO, true, false><<<grid, kBlock, 0, st>>>(

@@ -92,7 +92,8 @@ __global__ void __launch_bounds__(32) k_small_grad(const __grid_constant__ WfDev
 #pragma unroll
   for (int d = 0; d < 3; ++d) rt[d] = BF ? fma(wf.bf_w, pt.drt[d], r[d]) : r[d];
   Mo<NO, 2> mo;
-  orbitals<double, NO, 2>(wf, rt, mo);
+  const Tables tb{wf.shells, wf.mo_x2, wf.exp_tab};
+  orbitals<double, NO, 2>(wf, tb, rt, mo);
   double ai[NO];
   const double det = cofactors<NO>(g, mo.phi, a, n, i0, ai);
   const double idet = recip3(det);
@@ -297,7 +298,7 @@ __global__ void __launch_bounds__(32) k_small_grad(const __grid_constant__ WfDev
       const ShellDev& sh = wf.shells[sh0];
       if (sh.atom != atom) break;
       double f, g1, f2, q;
-      radial<2>(wf, sh, sh0, gg, f, g1, f2, q);
+      radial<2>(wf, tb, sh, sh0, gg, f, g1, f2, q);
       const double t3 = radial_third(wf, sh, sh0, gg, f, q);
       const int row = sh.ao_first, na = sh.l == 0 ? 1 : 3, p0 = prim_start[row];
       double uu[3] = {0.0, 0.0, 0.0};
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(32) k_small_grad(const __grid_constant__ WfDev
           const double pf = sh.l == 0 ? f : gg.v[e] * f;
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            const double c = mo_coef(wf, row + e, m, 0.0);
+            const double c = mo_coef(wf, tb, row + e, m, 0.0);
             u = fma(c, ai[m], u);
             w0 = fma(c, bphi[m], w0);
 #pragma unroll

@@ -255,6 +255,13 @@ __device__ __forceinline__ void macc(f32x2& acc, f32x2 a, f32x2 b) { mac_x2(acc,
 __device__ __forceinline__ double settle(double a) { return a; }
 __device__ __forceinline__ f32x2 settle(f32x2 a) { return normalize_x2(a); }
 
+// where the orbital tables are read (global or shared memory)
+struct Tables {
+  const ShellDev* shells;
+  const float2* mo_x2;     // pairs of FP32
+  const float* exp_tab;
+};
+
 template <typename U>
 struct Geo {  // an electron's displacement from a nucleus
   U v[3], r2, rho, irho, ir2;
@@ -284,8 +291,8 @@ __device__ __forceinline__ void geometry(const double p[3], const double* R, boo
 
 // f, g1 = f'/rho, f2 = f'' and q = (f2 - g1)/rho^2 of a shell
 template <int MODE>
-__device__ __forceinline__ void radial(const WfDev& wf, const ShellDev& sh, int s, const Geo<double>& g, double& f,
-                                       double& g1, double& f2, double& q) {
+__device__ __forceinline__ void radial(const WfDev& wf, const Tables&, const ShellDev& sh, int s,
+                                       const Geo<double>& g, double& f, double& g1, double& f2, double& q) {
   const double* nak = wf.nak + (size_t)s * QMC_MAX_PRIM;
   if (sh.kind == 0) {
     const double z = sh.expo[0];
@@ -318,11 +325,11 @@ __device__ __forceinline__ void radial(const WfDev& wf, const ShellDev& sh, int 
   }
 }
 template <int MODE>
-__device__ __forceinline__ void radial(const WfDev& wf, const ShellDev& sh, int, const Geo<f32x2>& g, f32x2& f,
-                                       f32x2& g1, f32x2& f2, f32x2& q) {
+__device__ __forceinline__ void radial(const WfDev&, const Tables& tb, const ShellDev& sh, int, const Geo<f32x2>& g,
+                                       f32x2& f, f32x2& g1, f32x2& f2, f32x2& q) {
   if (sh.kind == 0) {
     const f32x2 z(sh.expo_f[0], sh.expo_lo[0]);
-    f = f32x2(sh.coef_f[0], sh.coef_lo[0]) * exp_x2(-(z * g.rho), wf.exp_tab);
+    f = f32x2(sh.coef_f[0], sh.coef_lo[0]) * exp_x2(-(z * g.rho), tb.exp_tab);
     for (int k = 0; k < sh.kn; ++k) f = f * g.rho;
     if (MODE) {
       const f32x2 h = g.irho * (float)sh.kn - z, hf = h * f;
@@ -334,7 +341,7 @@ __device__ __forceinline__ void radial(const WfDev& wf, const ShellDev& sh, int,
     f = f32x2(0.f);
     f32x2 t1(0.f), t2(0.f);
     for (int p = 0; p < sh.n_prim; ++p) {
-      const f32x2 e = exp_x2(-(f32x2(sh.expo_f[p], sh.expo_lo[p]) * g.r2), wf.exp_tab);
+      const f32x2 e = exp_x2(-(f32x2(sh.expo_f[p], sh.expo_lo[p]) * g.r2), tb.exp_tab);
       mac_x2(f, f32x2(sh.coef_f[p], sh.coef_lo[p]), e);
       if (MODE) {
         mac_x2(t1, f32x2(sh.c2a_f[p], sh.c2a_lo[p]), e);
@@ -352,16 +359,16 @@ __device__ __forceinline__ void radial(const WfDev& wf, const ShellDev& sh, int,
   }
 }
 
-__device__ __forceinline__ double mo_coef(const WfDev& wf, int row, int m, double) {
+__device__ __forceinline__ double mo_coef(const WfDev& wf, const Tables&, int row, int m, double) {
   return __ldg(wf.mo64c + (size_t)row * wf.n_mo + m);
 }
-__device__ __forceinline__ f32x2 mo_coef(const WfDev& wf, int row, int m, f32x2) {
-  const float2 c = __ldg(wf.mo_x2 + (size_t)row * wf.n_mo + m);
+__device__ __forceinline__ f32x2 mo_coef(const WfDev& wf, const Tables& tb, int row, int m, f32x2) {
+  const float2 c = tb.mo_x2[(size_t)row * wf.n_mo + m];
   return f32x2(c.x, c.y);
 }
 
 template <typename U, int NO, int MODE>
-__device__ __forceinline__ void orbitals(const WfDev& wf, const double p[3], Mo<NO, MODE>& out) {
+__device__ __forceinline__ void orbitals(const WfDev& wf, const Tables& tb, const double p[3], Mo<NO, MODE>& out) {
   constexpr int ND = MODE ? NO : 1, NH = MODE == 2 ? 6 : 1;
   constexpr bool kPair = std::is_same<U, f32x2>::value;
   U phi[NO], dm[ND][3], hm[ND][NH];
@@ -378,7 +385,7 @@ __device__ __forceinline__ void orbitals(const WfDev& wf, const double p[3], Mo<
   }
   Geo<U> g;
   for (int s = 0; s < wf.n_shell;) {
-    const int atom = wf.shells[s].atom;
+    const int atom = tb.shells[s].atom;
     geometry<MODE>(p, wf.atom_xyz[atom], wf.any_sto != 0, g);
 #pragma unroll
     for (int m = 0; m < NO; ++m) {
@@ -393,16 +400,16 @@ __device__ __forceinline__ void orbitals(const WfDev& wf, const double p[3], Mo<
       for (int d = 0; d < 3; ++d) p1[m][d] = p2[m][d] = zero;
     }
     for (; s < wf.n_shell; ++s) {  // the shells of this run of the atom
-      const ShellDev& sh = wf.shells[s];
+      const ShellDev& sh = tb.shells[s];
       if (sh.atom != atom) break;
       U f, g1 = zero, f2 = zero, q = zero;
-      radial<MODE>(wf, sh, s, g, f, g1, f2, q);
+      radial<MODE>(wf, tb, sh, s, g, f, g1, f2, q);
       const int row = sh.ao_first;
       if (sh.l == 0) {
         if (MODE == 1) q = f2 + g1 * U(2.0f);
 #pragma unroll
         for (int m = 0; m < NO; ++m) {
-          const U c = mo_coef(wf, row, m, zero);
+          const U c = mo_coef(wf, tb, row, m, zero);
           macc(s0[m], c, f);
           if (MODE) {
             macc(s1[m], c, g1);
@@ -415,7 +422,7 @@ __device__ __forceinline__ void orbitals(const WfDev& wf, const double p[3], Mo<
         for (int d = 0; d < 3; ++d)
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            const U c = mo_coef(wf, row + d, m, zero);
+            const U c = mo_coef(wf, tb, row + d, m, zero);
             macc(p0[m][d], c, f);
             if (MODE) {
               macc(p1[m][d], c, g1);

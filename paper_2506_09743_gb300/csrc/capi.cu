@@ -471,7 +471,7 @@ qmc_status build_tables(qmc_wf* wf) {
     }
     pass_used.push_back(used);
     d.n_pass = (int)pass_used.size();
-    std::vector<int> lists, lists2;  // shell lists in four and in two parts per row
+    std::vector<int> lists, lists2, lists3;  // shell lists in four, two and three parts per row
     if (d.n_pass > kMaxTcPass) return fail(QMC_ERR_UNSUPPORTED, "too many AO passes");
     for (int p = 0; p < d.n_pass; ++p) {
       d.pass_zero[p] = ~pass_used[p];
@@ -520,12 +520,16 @@ qmc_status build_tables(qmc_wf* wf) {
       std::swap(lists, lists2);
       split(2, d.part2_off[p]);
       std::swap(lists, lists2);
+      std::swap(lists, lists3);
+      split(3, d.part3_off[p]);
+      std::swap(lists, lists3);
     }
     // the two-part lists follow the four-part ones
     for (int p = 0; p < d.n_pass; ++p)
       for (int q = 0; q < 3; ++q) d.part2_off[p][q] += d.n_shell;
     tc_shells = lists;
     tc_shells.insert(tc_shells.end(), lists2.begin(), lists2.end());
+    tc_shells.insert(tc_shells.end(), lists3.begin(), lists3.end());
   }
   if (d.gen_x2)
     for (const ShellDev& q : shells)
@@ -556,6 +560,14 @@ qmc_status build_tables(qmc_wf* wf) {
   // ---- small-molecule path (small_eval.cuh): MO rows in canonical shell order,
   // scaled exponents, 2^(j/2048)
   bool all_sp = true;
+  d.oz_pk_prims = 0;
+  for (const ShellDev& q : shells) {
+    if (q.kind != 1 || q.canon == 0) {
+      d.oz_pk_prims = 0;
+      break;
+    }
+    d.oz_pk_prims += q.n_prim;
+  }
   d.any_sto = 0;
   std::vector<double> nak((size_t)d.n_shell * QMC_MAX_PRIM, 0.0);
   for (int q = 0; q < d.n_shell; ++q) {

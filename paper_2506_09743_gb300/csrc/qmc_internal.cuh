@@ -103,6 +103,7 @@ struct WfDev {
   // {|AO value|, |kinetic value| = x + |grad J| y} over bins of r^2 (oz_bound_bin);
   // nullptr: the kernel bounds every shell instead
   const float4* oz_bound;
+  int oz_pk_prims;         // shell primitives when every shell is a complete Gaussian s, p or d shell (k_ao_mo_oz_pk), else 0
   int tc_value;            // 1: the FP32X2 form's Metropolis value path runs k_ao_mo_tc (FP32 AOs)
   int det_x2;              // 1: the FP32X2 form's determinant stage runs k_det_x2 (pairs of FP32), 0: k_det (FP64)
   const float* exp_tab;    // [64][2] 2^(j/64) as pairs: exp of the FP32X2 form
@@ -146,13 +147,14 @@ struct WfDev {
   // tc_shells[part2_off[p][q] .. part2_off[p][q+1]) (k_ao_mo_oz with two
   // thread groups).
   const int* ao_col;     // [n_ao]
-  const int* tc_shells;  // [2][n_shell]
+  const int* tc_shells;  // [3][n_shell]
   long long wait_cycles; // budget of a bounded device wait, SM clock cycles (qmc_set_wait_limit)
   int k_pad;             // n_pass * kTcPass (0 when the form has no tensor-core stage)
   int n_pass;
   unsigned pass_zero[kMaxTcPass];
   int part_off[kMaxTcPass][5];
   int part2_off[kMaxTcPass][3];
+  int part3_off[kMaxTcPass][4];  // three parts: offsets from tc_shells + 2 n_shell (k_ao_mo_oz_pk)
 };
 
 struct Workspace {
@@ -344,6 +346,10 @@ bool oz_supported(const WfDev& wf);
 int oz_groups(const WfDev& wf, int nch);  // thread groups of k_ao_mo_oz (1 or 2)
 cudaError_t launch_ao_mo_oz(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
                             int nch, int* err_flag, int* err_wf, cudaStream_t st);
+// two rows per thread in packed FP32 instructions
+bool oz_pk_supported(const WfDev& wf, int nch);
+cudaError_t launch_ao_mo_oz_pk(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
+                               int nch, int* err_flag, int* err_wf, cudaStream_t st);
 cudaError_t launch_ao_mo_x2(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
                             int nch, cudaStream_t st);
 cudaError_t launch_ao_mo_tc(const WfDev& wf, int prec, const double* walkers, int64_t W, int64_t ldw,

@@ -14,8 +14,8 @@
 // The kernel has 36% fewer instructions than k_ao_mo_oz, and what is left waits on
 // dependent FMAs and the FMA pipe: 2, 3 and 4 parts, that is as many warps per
 // scheduler, issue 38%, 49% and 53% of the time and took 3.59, 3.11 and 3.14 ms
-// (k_ao_mo_oz 3.39 ms).  A primitive's constants are kept in
-// shared memory in both lanes of a packed word (64 bytes, four broadcast loads).
+// (k_ao_mo_oz 3.39 ms).  A primitive's constants are kept in shared memory in
+// both lanes of a packed word (64 bytes, four broadcast loads).
 // The digits are stored negated (their remainders then come from one FMA), and
 // so are the MO digits of the B stack: the products are the same.
 #include <algorithm>
@@ -115,7 +115,20 @@ __global__ void __launch_bounds__(kPkThreads, 1)
   uint32_t commits = 0, iter = 0;
   double nr[2][3];
   float ng[2][3];
-  auto fetch = [&](int64_t t) {
+  // (walker block, electron) of the next tile, advanced without divisions
+  const unsigned n_el = (unsigned)wf.n_elec, first = blockIdx.x + grp * gridDim.x;
+  int64_t next_wb = first / n_el;
+  unsigned next_i = first % n_el;
+  const unsigned step_wb = kPkGroups * gridDim.x / n_el, step_i = kPkGroups * gridDim.x % n_el;
+  auto advance = [&]() {
+    next_wb += step_wb;
+    next_i += step_i;
+    if (next_i >= n_el) {
+      next_i -= n_el;
+      ++next_wb;
+    }
+  };
+  auto fetch = [&]() {
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
@@ -123,9 +136,8 @@ __global__ void __launch_bounds__(kPkThreads, 1)
         nr[q][d] = 0.0;
         ng[q][d] = 0.f;
       }
-    if (t >= n_tiles) return;
-    const int ti = (int)(t % wf.n_elec);
-    const int64_t tw = (t / wf.n_elec) * kRows + rp;
+    const int64_t tw = next_wb * kRows + rp;  // past W past the last tile
+    const int ti = (int)next_i;
 #pragma unroll
     for (int q = 0; q < 2; ++q)
       if (tw + q * kPkPairs < W)
@@ -136,11 +148,11 @@ __global__ void __launch_bounds__(kPkThreads, 1)
         }
   };
   const int64_t tile_step = (int64_t)kPkGroups * gridDim.x;
-  fetch(blockIdx.x + (int64_t)grp * gridDim.x);
+  fetch();
   for (int64_t tile = blockIdx.x + (int64_t)grp * gridDim.x; tile < n_tiles; tile += tile_step, ++iter) {
     int* rowe = rowe_buf + (iter & 1u) * 2 * kRows;
-    const int i = (int)(tile % wf.n_elec);
-    const int64_t wb = tile / wf.n_elec;
+    const int i = (int)next_i;
+    const int64_t wb = next_wb;
     double r[2][3];
     float gq[2][3];
 #pragma unroll
@@ -338,7 +350,8 @@ __global__ void __launch_bounds__(kPkThreads, 1)
       oz_poison<NCH>(tile, tile_step, n_tiles, wf.n_elec, rp + kPkPairs, part, kPkParts, W, mo_out, nmp, ldm);
       break;
     }
-    fetch(tile + tile_step);
+    advance();
+    fetch();
     // ---- 3. epilogue
     // (six warps: two quarters of the rows have two warps, two have one)
     const int lw = warp % (kPkGT / 32);

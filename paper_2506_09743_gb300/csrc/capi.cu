@@ -97,7 +97,7 @@ size_t workspace_bytes(const qmc_wf* wf, int64_t W) {
   b += align256((size_t)N * 2 * mo_row_pad(wf->dev.n_mo, tc) * ldm * sizeof(double));  // MO channels (FP64)
   b += align256(3 * N * ldm * sizeof(double));         // proposals
   b += 2 * align256(ldm * sizeof(double));             // lp, lp_new
-  b += align256(sizeof(uint64_t));                     // step counter
+  b += align256(2 * sizeof(uint64_t));                     // step counter
   b += align256(sizeof(int));                          // device error flag
   return b;
 }
@@ -116,7 +116,7 @@ Workspace carve(const qmc_wf* wf, void* base, int64_t W, int** err_flag) {
   ws.prop = reinterpret_cast<double*>(p); p += align256(3 * N * ws.ldm * sizeof(double));
   ws.lp = reinterpret_cast<double*>(p); p += align256(ws.ldm * sizeof(double));
   ws.lp_new = reinterpret_cast<double*>(p); p += align256(ws.ldm * sizeof(double));
-  ws.ctr = reinterpret_cast<uint64_t*>(p); p += align256(sizeof(uint64_t));
+  ws.ctr = reinterpret_cast<uint64_t*>(p); p += align256(2 * sizeof(uint64_t));
   *err_flag = reinterpret_cast<int*>(p);
   return ws;
 }
@@ -1132,7 +1132,7 @@ qmc_status qmc_local_energy_host(qmc_wf* wf, const double* walkers, int64_t n_wa
 }
 
 // Metropolis steps as a CUDA graph: one step (proposal, value path on the
-// proposals, acceptance, step-counter advance) is captured once on the
+// proposals, acceptance; both advance the step counter) is captured once on the
 // wavefunction's capture stream and replayed n_steps times on st, so a
 // launch-bound chain (small walker counts) pays one graph launch per step
 // instead of five to seven kernel launches.  The step index comes from a
@@ -1161,7 +1161,6 @@ static qmc_status sample_graph(qmc_wf* wf, double* walkers, int64_t W, int64_t l
   if (!s)
     s = launch_status(
         launch_accept(wf->dev, walkers, W, ldw, ws, seed, first_walker, step_offset, ws.ctr, n_accept, cs), "accept");
-  if (!s) s = launch_status(launch_step_advance(ws.ctr, cs), "step counter");
   cudaGraph_t graph = nullptr;
   cudaError_t e = cudaStreamEndCapture(cs, &graph);
   if (s || e != cudaSuccess || !graph) {  // not capturable here: the plain loop runs instead
@@ -1176,7 +1175,7 @@ static qmc_status sample_graph(qmc_wf* wf, double* walkers, int64_t W, int64_t l
     cudaGetLastError();
     return QMC_OK;
   }
-  e = cudaMemsetAsync(ws.ctr, 0, sizeof(uint64_t), st);
+  e = cudaMemsetAsync(ws.ctr, 0, 2 * sizeof(uint64_t), st);
   for (int t = 0; e == cudaSuccess && t < n_steps; ++t) e = cudaGraphLaunch(exec, st);
   cudaGraphExecDestroy(exec);  // freed once the launched replays complete
   if (e != cudaSuccess) return cuda_fail(e, "step graph launch");

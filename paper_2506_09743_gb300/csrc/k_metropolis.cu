@@ -8,7 +8,11 @@
 // the acceptance uniform.  Both kernels regenerate their numbers from the
 // counter, so nothing random is stored between them.  The step index is
 // gstep plus, when gctr is not null, a device counter: a CUDA graph of one
-// step is then replayed with the counter advanced by a one-thread kernel.
+// step is then replayed, and the kernels advance the counter themselves: the
+// proposal reads gctr[0] and writes gctr[1] = gctr[0] + 1, the acceptance reads
+// gctr[1] and writes it back to gctr[0] (each word has one writer, and its
+// readers run in the kernel after it).  A one-thread kernel of its own took
+// 1.5 us and a launch a step.
 #include <cmath>
 #include <mutex>
 #include <vector>
@@ -67,10 +71,13 @@ cudaError_t box_muller_tables(BmTables* t) {
 __global__ void __launch_bounds__(128) k_propose(int n3, const double* __restrict__ walkers, int64_t W, int64_t ldw,
                                                  double* __restrict__ prop, int64_t ldm, double step, uint64_t seed,
                                                  uint64_t first_walker, uint64_t gstep,
-                                                 const unsigned long long* __restrict__ gctr) {
+                                                 unsigned long long* __restrict__ gctr) {
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= W) return;
-  if (gctr) gstep += *gctr;
+  if (gctr) {
+    gstep += gctr[0];
+    if (w == 0 && blockIdx.y == 0) gctr[1] = gctr[0] + 1ull;
+  }
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   const uint32_t wi = (uint32_t)(first_walker + (uint64_t)w);
   const int j = blockIdx.y;
@@ -88,11 +95,14 @@ __global__ void __launch_bounds__(128) k_accept(int n3, double* __restrict__ wal
                                                 const double* __restrict__ prop, int64_t ldm,
                                                 double* __restrict__ lp, const double* __restrict__ lp_new,
                                                 uint64_t seed, uint64_t first_walker, uint64_t gstep,
-                                                const unsigned long long* __restrict__ gctr,
+                                                unsigned long long* __restrict__ gctr,
                                                 int64_t* __restrict__ n_accept) {
   const int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (w >= W) return;
-  if (gctr) gstep += *gctr;
+  if (gctr) {
+    gstep += gctr[1] - 1ull;
+    if (w == 0) gctr[0] = gctr[1];
+  }
   const uint32_t wi = (uint32_t)(first_walker + (uint64_t)w);
   const int nblk = (n3 + 3) / 4;
   const u4 x = philox4x32_10(u4{(uint32_t)nblk, wi, (uint32_t)gstep, (uint32_t)(gstep >> 32)}, (uint32_t)seed,
@@ -126,9 +136,6 @@ __global__ void __launch_bounds__(128) k_init_walkers(InitSpec spec, int64_t W, 
   }
 }
 
-// the step counter of a replayed step graph: one more step done
-__global__ void k_step_advance(unsigned long long* ctr) { *ctr += 1ull; }
-
 // sum of the per-walker acceptance counts into out[0] (fixed order)
 __global__ void k_sum_counts(const int64_t* __restrict__ c, int64_t W, double* __restrict__ out) {
   __shared__ long long red[256];
@@ -156,28 +163,22 @@ cudaError_t launch_sum_counts(const int64_t* counts, int64_t W, double* out, cud
 }
 
 cudaError_t launch_propose(const WfDev& wf, const double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
-                           double step, uint64_t seed, uint64_t first_walker, uint64_t gstep, const uint64_t* gctr,
+                           double step, uint64_t seed, uint64_t first_walker, uint64_t gstep, uint64_t* gctr,
                            cudaStream_t st) {
   if (W == 0) return cudaSuccess;
   const dim3 grid((unsigned)((W + 127) / 128), (unsigned)((3 * wf.n_elec + 3) / 4));
-  k_propose<<<grid, 128, 0, st>>>(3 * wf.n_elec, walkers, W, ldw, ws.prop, ws.ldm, step,
-                                                          seed, first_walker, gstep,
-                                                          reinterpret_cast<const unsigned long long*>(gctr));
-  return cudaGetLastError();
-}
-
-cudaError_t launch_step_advance(uint64_t* gctr, cudaStream_t st) {
-  k_step_advance<<<1, 1, 0, st>>>(reinterpret_cast<unsigned long long*>(gctr));
+  k_propose<<<grid, 128, 0, st>>>(3 * wf.n_elec, walkers, W, ldw, ws.prop, ws.ldm, step, seed, first_walker, gstep,
+                                  reinterpret_cast<unsigned long long*>(gctr));
   return cudaGetLastError();
 }
 
 cudaError_t launch_accept(const WfDev& wf, double* walkers, int64_t W, int64_t ldw, const Workspace& ws,
-                          uint64_t seed, uint64_t first_walker, uint64_t gstep, const uint64_t* gctr,
+                          uint64_t seed, uint64_t first_walker, uint64_t gstep, uint64_t* gctr,
                           int64_t* n_accept, cudaStream_t st) {
   if (W == 0) return cudaSuccess;
   k_accept<<<(unsigned)((W + 127) / 128), 128, 0, st>>>(3 * wf.n_elec, walkers, W, ldw, ws.prop, ws.ldm, ws.lp,
                                                          ws.lp_new, seed, first_walker, gstep,
-                                                         reinterpret_cast<const unsigned long long*>(gctr), n_accept);
+                                                         reinterpret_cast<unsigned long long*>(gctr), n_accept);
   return cudaGetLastError();
 }
 

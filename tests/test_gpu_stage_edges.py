@@ -17,7 +17,7 @@ import pytest
 import torch
 
 import qmc_inputs as qi
-from gpu_common import fp64_check, gated_check, oracle_reference
+from gpu_common import fp32ao_check, fp64_check, gated_check, oracle_reference
 from oracle import qmc_oracle as O
 
 pytestmark = pytest.mark.gpu
@@ -158,6 +158,29 @@ def test_packed_rows_match_single_rows(pkg, shells, n_mo):
         assert torch.isfinite(la).sum() >= W - 2
     a.close()
     b.close()
+
+
+# -- TF32 AO stage: two rows per thread, shells of every kind
+@pytest.mark.parametrize("shells", ["ssp", "sspd", "sPDf"])
+@pytest.mark.parametrize("sto", [False, True])
+def test_tf32_rows_of_any_shell(pkg, shells, sto):
+    mol = _mol(5, 4, shells, 6, 3, sto=sto)
+    r = qi.walkers(mol, 259, seed=9)
+    E, lp, sens = oracle_reference(mol, r)
+    wf = pkg.Wavefunction(mol, precision="mixed_tf32")
+    full = None
+    for W in (259, 129, 128, 65, 64, 63, 1):
+        e, l = wf.local_energy(_x(r, 1), n_walkers=W)
+        torch.cuda.synchronize()
+        fp32ao_check(e.cpu().numpy(), E[:W], sens[:W])
+        full = (e, l) if full is None else full
+        assert torch.equal(e, full[0][:W]) and torch.equal(l, full[1][:W])  # a row does not depend on the batch
+    # the value path (a chain of no steps returns log|Psi| of where it stands)
+    x, lps = _x(r, 1), torch.empty(259, dtype=torch.float64, device="cuda")
+    wf.sample(x, 0, 0.3, 5, n_walkers=259, log_psi=lps)
+    torch.cuda.synchronize()
+    assert np.all(np.abs(lps.cpu().numpy() - lp) <= 128 * 2.0 ** -24 * sens * np.maximum(1.0, np.abs(lp)))
+    wf.close()
 
 
 # -- gradient rows: tiles of 32 walkers, chunks of AOs and radial derivatives

@@ -339,7 +339,7 @@ qmc_status build_tables(qmc_wf* wf) {
     const double df = dfact(2 * kx - 1) * dfact(2 * ky - 1) * dfact(2 * kz - 1);
     ShellDev sh{};
     sh.atom = atom;
-    sh.kind = kind;
+    sh.kind = (short)kind;
     sh.kn = kind == 0 ? kn : 0;
     sh.l = l;
     sh.n_prim = s1 - s0;
@@ -560,6 +560,7 @@ qmc_status build_tables(qmc_wf* wf) {
   // ---- small-molecule path (small_eval.cuh): MO rows in canonical shell order,
   // scaled exponents, 2^(j/2048)
   bool all_sp = true;
+  std::vector<int> small_row(nao);  // row of each AO in the small-molecule tables
   d.oz_pk_prims = 0;
   for (const ShellDev& q : shells) {
     if (q.kind != 1 || q.canon == 0) {
@@ -571,14 +572,33 @@ qmc_status build_tables(qmc_wf* wf) {
   d.any_sto = 0;
   std::vector<double> nak((size_t)d.n_shell * QMC_MAX_PRIM, 0.0);
   for (int q = 0; q < d.n_shell; ++q) {
-    all_sp = all_sp && (shells[q].canon == 1 || shells[q].canon == 2);
+    // s shells, and p shells of distinct functions (all three, or fewer where
+    // their exponents differ); rows x before y before z
+    ShellDev& sh = shells[q];
+    sh.p_mask = 0;
+    bool distinct = sh.l <= 1 && (sh.l == 1 || sh.n_ao == 1);
+    auto axis = [&](int b) { return (ao_pow[b] & 15) ? 0 : ((ao_pow[b] >> 4) & 15) ? 1 : 2; };
+    if (sh.l == 1)
+      for (int k = 0; k < sh.n_ao; ++k) {
+        distinct = distinct && !((sh.p_mask >> axis(sh.ao_first + k)) & 1);
+        sh.p_mask = (short)(sh.p_mask | 1 << axis(sh.ao_first + k));
+      }
+    for (int k = 0; k < sh.n_ao; ++k) {
+      int rank = 0;
+      if (sh.l == 1)
+        for (int j = 0; j < sh.n_ao; ++j) rank += axis(sh.ao_first + j) < axis(sh.ao_first + k);
+      small_row[sh.ao_first + k] = sh.ao_first + (sh.l == 1 ? rank : k);
+      // the pair tables' rows are in the order of x2_row
+      if (d.gen_x2 && small_row[sh.ao_first + k] != x2_row[sh.ao_first + k]) distinct = false;
+    }
+    all_sp = all_sp && distinct;
     if (shells[q].kind == 0) d.any_sto = 1;
     for (int k = 0; k < shells[q].n_prim; ++k)
       nak[(size_t)q * QMC_MAX_PRIM + k] = (double)(-2048.0L * (long double)shells[q].expo[k] / 0.6931471805599453094L);
   }
   std::vector<double> mo64c((size_t)nao * nmo);
   for (int b = 0; b < nao; ++b)
-    for (int m = 0; m < nmo; ++m) mo64c[(size_t)x2_row[b] * nmo + m] = mo64[(size_t)b * nmo + m];
+    for (int m = 0; m < nmo; ++m) mo64c[(size_t)small_row[b] * nmo + m] = mo64[(size_t)b * nmo + m];
   // (the table of powers is the same for every wavefunction: built once, since
   // qmc_set_params rebuilds the tables at every optimisation step)
   static const std::vector<double> exp2_tab = [] {
@@ -592,7 +612,7 @@ qmc_status build_tables(qmc_wf* wf) {
     for (int k = 0; k < q.n_ao; ++k)
       for (int p = 0; p < q.n_prim; ++p)
         prim_val[h.prim_start[q.ao_first + k] + p] =
-            h.prim_start[q.ao_first] + (x2_row[q.ao_first + k] - q.ao_first) * q.n_prim + p;
+            h.prim_start[q.ao_first] + (small_row[q.ao_first + k] - q.ao_first) * q.n_prim + p;
   d.log_w0 = ndet == 1 ? std::log(std::fabs(h.det_w[0])) : 0.0;
 
   // ---- determinants: unique excitation records per spin.  The expansion is
@@ -751,7 +771,7 @@ qmc_status build_tables(qmc_wf* wf) {
       {mo_oz.data(), sizeof(uint16_t) * mo_oz.size()},  {oz_bnd.data(), sizeof(float) * oz_bnd.size()},
       {order.data(), sizeof(int) * order.size()},        {mo_x2n.data(), sizeof(float) * mo_x2n.size()},
       {mo64c.data(), sizeof(double) * mo64c.size()},     {nak.data(), sizeof(double) * nak.size()},
-      {exp2_tab.data(), sizeof(double) * exp2_tab.size()}, {x2_row.data(), sizeof(int) * nao},
+      {exp2_tab.data(), sizeof(double) * exp2_tab.size()}, {small_row.data(), sizeof(int) * nao},
       {prim_val.data(), sizeof(int) * prim_val.size()}};
   size_t total = 0;
   for (auto& p : parts) total += align256(p.second);

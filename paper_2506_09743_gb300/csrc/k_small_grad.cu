@@ -300,26 +300,27 @@ __global__ void __launch_bounds__(32) k_small_grad(const __grid_constant__ WfDev
       double f, g1, f2, q;
       radial<2>(wf, tb, sh, sh0, gg, f, g1, f2, q);
       const double t3 = radial_third(wf, sh, sh0, gg, f, q);
-      const int row = sh.ao_first, na = sh.l == 0 ? 1 : 3, p0 = prim_start[row];
+      const int row = sh.ao_first, mask = sh.l == 0 ? 1 : sh.p_mask, p0 = prim_start[row];
       double uu[3] = {0.0, 0.0, 0.0};
 #pragma unroll
       for (int e = 0; e < 3; ++e)
-        if (e < na) {
+        if ((mask >> e) & 1) {
+          const int k = e == 0 ? 0 : __popc(mask & ((1 << e) - 1));  // its AO within the shell
           double w0 = 0.0, w1[3] = {0.0, 0.0, 0.0}, u = 0.0;
           const double pf = sh.l == 0 ? f : gg.v[e] * f;
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            const double c = mo_coef(wf, tb, row + e, m, 0.0);
+            const double c = mo_coef(wf, tb, row + k, m, 0.0);
             u = fma(c, ai[m], u);
             w0 = fma(c, bphi[m], w0);
 #pragma unroll
             for (int d = 0; d < 3; ++d) w1[d] = fma(c, bd[m][d], w1[d]);
-            put(off_c + (row + e) * NO + m, pf * ai[m]);
+            put(off_c + (row + k) * NO + m, pf * ai[m]);
           }
           uu[e] = u;
           if (sh.kind == 0) {
             const double nq = (double)(sh.kn + sh.l + 1) + 0.5;
-            put(p0 + e, u * pf * (nq * recip3(sh.expo[0]) - gg.rho));
+            put(p0 + k, u * pf * (nq * recip3(sh.expo[0]) - gg.rho));
           }
           if (sh.l == 0) {
             sg0 = fma(g1, w0, sg0);
@@ -354,7 +355,8 @@ __global__ void __launch_bounds__(32) k_small_grad(const __grid_constant__ WfDev
                               ((0.75 + 0.5 * sh.l) * recip3(sh.expo[p]) - gg.r2);
 #pragma unroll
           for (int e = 0; e < 3; ++e)
-            if (e < na) put(p0 + e * sh.n_prim + p, uu[e] * (sh.l == 0 ? term : gg.v[e] * term));
+            if ((mask >> e) & 1)
+              put(p0 + __popc(mask & ((1 << e) - 1)) * sh.n_prim + p, uu[e] * (sh.l == 0 ? term : gg.v[e] * term));
         }
       }
     }

@@ -37,7 +37,10 @@ constexpr int kMaxTcPass = 16;   // passes (QMC_MAX_AO columns, gaps of < kMaxSh
 // and primitives).  Radial normalisation and contraction coefficients are
 // folded into coef; the per-AO angular factor is folded into the MO table.
 struct ShellDev {
-  int atom, kind, kn, l;
+  int atom;
+  short kind;
+  short p_mask;  // p shell: bit d set where it holds the function along d
+  int kn, l;
   int n_prim, ao_first, n_ao;
   int canon;  // 1 + l for a complete Cartesian s, p or d shell, else 0 (FP32X2 form:
               // its MO table rows are in the canonical order s; x, y, z; xx, xy, xz, yy, yz, zz)
@@ -122,7 +125,7 @@ struct WfDev {
   const uint32_t* mo_tc_hi;
   const uint32_t* mo_tc_lo;
   // small-molecule path (small_eval.cuh): 1 when it serves this wavefunction
-  // (one determinant, <= 8 electrons, <= 4 per spin, complete s and p shells);
+  // (one determinant, <= 8 electrons, <= 4 per spin, s and p shells);
   // MO table rows in canonical shell order, -2048 alpha / ln 2 per shell and
   // primitive, 2^(j/2048), whether any shell is a Slater function, log|d_0|
   int small;

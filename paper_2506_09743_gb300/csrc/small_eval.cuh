@@ -1,5 +1,5 @@
 // Device code of the small-molecule path: one determinant, at most 8
-// electrons (4 per spin), complete s and p shells, with or without backflow.
+// electrons (4 per spin), s and p shells, with or without backflow.
 // One lane per electron, 32 / N walkers per warp.
 //
 // What bounds these kernels is the FP64 pipe: a warp-wide FP64 instruction
@@ -418,17 +418,23 @@ __device__ __forceinline__ void orbitals(const WfDev& wf, const Tables& tb, cons
         }
       } else {
         if (MODE == 1) q = f2 + g1 * U(4.0f);
+        // (the functions that the shell holds: all three, or fewer where the
+        // exponents of x, y and z differ, as after an optimisation step)
+        int r = row;
 #pragma unroll
-        for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 3; ++d) {
+          if (!((sh.p_mask >> d) & 1)) continue;
 #pragma unroll
           for (int m = 0; m < NO; ++m) {
-            const U c = mo_coef(wf, tb, row + d, m, zero);
+            const U c = mo_coef(wf, tb, r, m, zero);
             macc(p0[m][d], c, f);
             if (MODE) {
               macc(p1[m][d], c, g1);
               macc(p2[m][d], c, q);
             }
           }
+          ++r;
+        }
       }
     }
     U dd[6];

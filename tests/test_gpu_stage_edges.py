@@ -213,3 +213,57 @@ def test_mean_and_variance_around_the_chunks(pkg, W):
     assert abs(m - e.mean()) <= 1e-10 * top
     assert abs(v - e.var()) <= 1e-8 * e.var() + 1e-10 * top * top
     wf.close()
+
+
+# -- small molecules: p functions held by shells of their own (as after an optimisation step)
+@pytest.mark.parametrize("n_up,n_down", [(1, 1), (3, 2), (4, 4)])
+@pytest.mark.parametrize("sto", [False, True])
+@pytest.mark.parametrize("precision,w", [("fp64", 0.0), ("fp64", 0.1), ("fp32x2", 0.1)])
+def test_split_p_shells_match_whole_ones(pkg, n_up, n_down, sto, precision, w):
+    """The functions of two p shells of a nucleus written alternately (x, x, y,
+    y, z, z) are six shells of one function: every sum keeps its order, so
+    energies, log|Psi|, chains and parameter gradients are the same bit for bit.
+    (The forces add the functions' terms in another order: 1e-12 of the largest.)"""
+    mol = dataclasses.replace(_mol(n_up, n_down, "spp", max(n_up, n_down) + 1, n_prim=2, sto=sto), backflow_w=w)
+    xyz = [int(np.argmax(k[:3])) for k in mol.ao_pow]  # axis of a p function
+    order = []
+    for a in range(3):  # per nucleus: s, then two p shells in any order
+        b = 7 * a
+        sh = [sorted(range(b + 1, b + 4), key=lambda k: xyz[k]), sorted(range(b + 4, b + 7), key=lambda k: xyz[k])]
+        order.append([b] + sh[0] + sh[1])
+    def pick(idx):
+        n = np.diff(mol.ao_prim_start)
+        pr = np.concatenate([np.arange(mol.ao_prim_start[k], mol.ao_prim_start[k + 1]) for k in idx])
+        return dataclasses.replace(
+            mol, ao_atom=mol.ao_atom[idx], ao_kind=mol.ao_kind[idx], ao_pow=mol.ao_pow[idx],
+            ao_prim_start=np.concatenate([[0], np.cumsum(n[idx])]).astype(np.int32), prim_exp=mol.prim_exp[pr],
+            prim_coef=mol.prim_coef[pr], mo_coeff=mol.mo_coeff[idx]), pr
+    whole, pr_w = pick(np.concatenate(order))
+    split, pr_s = pick(np.concatenate([[o[0], o[1], o[4], o[2], o[5], o[3], o[6]] for o in order]))
+    x = _x(qi.walkers(mol, 45, seed=12), 2)
+    a, b = pkg.Wavefunction(whole, precision=precision), pkg.Wavefunction(split, precision=precision)
+    ea, la = a.local_energy(x, n_walkers=45)
+    eb, lb = b.local_energy(x, n_walkers=45)
+    torch.cuda.synchronize()
+    assert torch.equal(ea, eb) and torch.equal(la, lb)
+    ya, yb = x.clone(), x.clone()
+    a.sample(ya, 5, 0.3, 13, n_walkers=45)
+    b.sample(yb, 5, 0.3, 13, n_walkers=45)
+    torch.cuda.synchronize()
+    assert torch.equal(ya, yb)
+    if precision == "fp64":
+        _, _, ga, fa = a.energy_grad(x, n_walkers=45)
+        _, _, gb, fb = b.energy_grad(x, n_walkers=45)
+        ga, gb = ga.cpu().numpy(), gb.cpu().numpy()
+        n = mol.prim_exp.size
+        ta, tb = np.empty(n), np.empty(n)
+        ta[pr_w], tb[pr_s] = ga[:n], gb[:n]
+        assert np.array_equal(ta, tb)
+        m = mol.mo_coeff.size
+        ca, cb = np.empty(mol.mo_coeff.shape), np.empty(mol.mo_coeff.shape)
+        ca[np.concatenate(order)] = ga[n:n + m].reshape(ca.shape)
+        cb[np.concatenate([[o[0], o[1], o[4], o[2], o[5], o[3], o[6]] for o in order])] = gb[n:n + m].reshape(cb.shape)
+        assert np.array_equal(ca, cb)
+        assert np.abs((fa - fb).cpu().numpy()).max() <= 1e-12 * max(1.0, float(fa.abs().max()))
+    a.close()
+    b.close()

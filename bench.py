@@ -45,9 +45,9 @@ FP64_PEAK_TFLOPS = 152 * 4 * 2.07e9 / 1e12  # 152 SMs x 2 DFMA/clk x 2 flop x 2.
 # mixed_tf32 and FP64 forms), from an ncu capture of that kernel on 131,072 CO walkers (418.6 MB per
 # launch); set to None whenever the kernel changes.
 DET_TRAFFIC_BYTES_PER_WALKER = (414.384128e6 + 4.216064e6) / 131072
-# DRAM bytes (read + write) per walker of the k_ao_mo_oz launch, from an ncu capture of that kernel on
-# 131,072 CO walkers (66.3 MB read, 409.0 MB written per launch); None whenever the kernel changes.
-OZ_TRAFFIC_BYTES_PER_WALKER = (66.262016e6 + 408.966912e6) / 131072
+# DRAM bytes (read + write) per walker of the k_ao_mo_oz_pk launch, from an ncu capture of that kernel on
+# 131,072 CO walkers (66.3 MB read, 406.7 MB written per launch); None whenever the kernel changes.
+OZ_TRAFFIC_BYTES_PER_WALKER = (66.336256e6 + 406.659072e6) / 131072
 # DRAM bytes (read + write) per walker of the k_det_x2 launch (FP32X2 determinant stage), from an ncu
 # capture of that kernel on 131,072 CO walkers; None whenever the kernel changes (the last capture,
 # 414.4 MB read and 1.2 MB written, was of the six-blocks-per-SM build).
@@ -223,7 +223,7 @@ def general_eloc_ops(mol) -> dict:
 
 
 def oz_stage_alu_ops(mol) -> float:
-    """Algorithmic FP32/ALU operations per walker of k_ao_mo_oz, the FP32X2
+    """Algorithmic FP32/ALU operations per walker of k_ao_mo_oz and k_ao_mo_oz_pk, the FP32X2
     AO stage with the contraction on the tensor cores.  Per electron: per
     Gaussian primitive of each shell -alpha rho^2 (7), the exponential (69)
     and three pair multiply-accumulates for the value and the two kinetic
@@ -457,7 +457,7 @@ def run_secondary(device, stream, barrier, flush, rates=None):
             wf = Wavefunction(mol, precision=form, device=device)
             out[f"{name}_{form}_walker_evals_per_s"] = rate(wf, x, W)
             if name == "li2" and form == "fp64":
-                # the general kernel's FP64 roofline: formula flops, and with
+                # FP64 roofline in the general kernel's formula flops, and with
                 # the special functions at their measured FMA equivalents
                 ops = general_eloc_ops(mol)
                 ms = 1e3 * W / out[f"{name}_{form}_walker_evals_per_s"]
@@ -469,12 +469,13 @@ def run_secondary(device, stream, barrier, flush, rates=None):
                           + ops["div"] * f / rates["fp64_recip_per_s"])
                     eq = (ops["flops"] + 2.0 * sp) * W / (ms / 1e3) / 1e12
                 out["li2_eloc_roofline"] = {
-                    "kernel": "k_eloc_general<6, 3>", "bound": "alu", "kernel_ms": ms, "unit": "TFLOP/s (FP64)",
+                    "kernel": "k_small_energy<6, 3>", "bound": "alu", "kernel_ms": ms, "unit": "TFLOP/s (FP64)",
                     "flops_per_walker": ops["flops"], "exp_per_walker": ops["exp"], "sqrt_per_walker": ops["sqrt"],
                     "div_per_walker": ops["div"], "achieved": fl, "peak": FP64_PEAK_TFLOPS,
                     "frac": fl / FP64_PEAK_TFLOPS, "achieved_with_special": eq,
                     "frac_with_special": None if eq is None else eq / FP64_PEAK_TFLOPS,
-                    "ops_model": "bench.general_eloc_ops; exp, sqrt and division at the measured FMA equivalents"}
+                    "ops_model": "bench.general_eloc_ops (the general kernel's formulas; k_small_energy needs fewer); exp, "
+                                 "sqrt and division at the measured FMA equivalents"}
             if name == "li2" and form == "fp64":
                 wf.energy_grad(x)
                 barrier()
@@ -858,7 +859,7 @@ def main():
     flops_det = det_stage_flops(mol) * W
     det_ms = float(stage_mixed[2])
     det_rate = flops_det / (det_ms / 1e3) / 1e12
-    roofline = {"kernel": "k_ao_mo_oz (AOs in pairs of FP32, exact digit-sliced contraction on tcgen05; FP32X2 form)",
+    roofline = {"kernel": "k_ao_mo_oz_pk (AOs in pairs of FP32, exact digit-sliced contraction on tcgen05; FP32X2 form)",
                 "bound": "alu", "achieved": oz_rate, "peak": FP32_PEAK_TOPS, "unit": "T FP32 ops/s",
                 "frac": oz_rate / FP32_PEAK_TOPS,
                 "traffic": None if OZ_TRAFFIC_BYTES_PER_WALKER is None else OZ_TRAFFIC_BYTES_PER_WALKER * W,
